@@ -238,6 +238,36 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// Two binary32 values in one 64-bit register, lower index in the low half: packed
+// operations issue once for both and round each as the scalar operation does.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // Sums of squares in binary32 double-single arithmetic: a value is the
 // unevaluated pair hi + lo.  ds_sq gives x^2 exactly (the FMA residual of the
 // rounded product), ds_add is Knuth's TwoSum followed by a fast

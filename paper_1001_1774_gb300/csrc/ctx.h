@@ -68,9 +68,9 @@ struct tvcs_ctx {
     bool own_stream = false;
     cudaStream_t cap_stream = nullptr;
     // device buffers
-    float* A = nullptr;            // binary32 A for the single-block-row product kernel (n <= 128)
-    bool use_q = false;            // products by clusters / reduced precision (k_products_q)
-    unsigned char *P0 = nullptr, *P1 = nullptr;   // storage planes of A on that path
+    float* A = nullptr;            // binary32 A (n <= 128; else, and in the other storages, P0 and P1 below)
+    bool use_q = false;            // products by clusters (k_products_q: n = 192, 256)
+    unsigned char *P0 = nullptr, *P1 = nullptr;   // storage planes of A
     float* rscale = nullptr;       // per-row scales of the fp8 storage
     float *f = nullptr, *u = nullptr, *w = nullptr, *lam = nullptr, *g = nullptr, *r = nullptr,
           *rhs = nullptr, *zeroN = nullptr;

@@ -1,78 +1,160 @@
 // Rows a6-a7: r = A x - y and g = A^T r in ONE pass over A (Xiao & Yang,
-// eq. (line): g_k = A^T (A u^k - f); two products per iteration, Sec. 3.1).
+// eq. (line): g_k = A^T (A u^k - f); two products per iteration, Sec. 3.1), for
+// images up to 128 x 128 and every storage of A (k_products_q.cu has the larger
+// ones and states the storages: binary32, bf16 hi + lo, fp8 e4m3 + bf16).
 //
-// Each block owns a contiguous range of rows of A (row-major binary32).  Thread
-// 0 streams the rows into a 3-stage shared-memory ring with bulk asynchronous
-// copies (TMA, non-tensor form, one mbarrier per stage; A is read once per
-// call, with an L2 evict-first hint), the first stages before the dependency
-// wait on the preceding kernel, together with an L2 prefetch of the next 1 MB
-// of the block's rows.  All 512 threads own fixed columns: for each
-// row they form the dot product with x (warp shuffles + one named barrier),
-// compute r_i = dot - y_i, and fold r_i * A_i into per-thread accumulators of
-// A^T r.  Row i's data is used twice from shared memory and read from HBM once,
-// so the algorithmic traffic is one pass over A.  Each block writes its partial
-// A^T r (N floats); with g_out set, a grid barrier (cooperative launch) follows
-// and every block sums its slice of the P partials in a fixed order
+// Each block owns a contiguous range of rows of A.  Thread 0 streams them into
+// a ring of NST stages of RS rows in shared memory with bulk asynchronous copies
+// (TMA, non-tensor form, one mbarrier per stage; A is read once per call, with
+// an L2 evict-first hint), the first stages before the dependency wait on the
+// preceding kernel, together with an L2 prefetch of the block's next rows.  A
+// thread owns fixed columns: it reads its columns of RB rows into registers
+// (decoded to binary32 once), forms the dot products with x (warp shuffles + one
+// named barrier for all RB rows), computes r_i = dot - y_i and folds r_i A_i into
+// its accumulators of A^T r from the same registers.  Each block writes its
+// partial A^T r (N floats); with g_out set, a grid barrier (cooperative launch)
+// follows and every block sums its slice of the P partials in a fixed order
 // (deterministic), otherwise a later kernel does.
 //
-// Shapes: 512 threads in RL row lanes of TPR = 512/RL threads; a thread holds V
-// float4 columns of x and of the accumulator (N = 4*TPR*V).  RS rows per stage,
-// 3 stages: one block per SM, and the grid leaves 16 SMs free for the u-solve.
+// What bounds it: HBM, once a row's step (stage wait, loads, warp shuffles, block
+// barrier, update; all warps in step) does not.  A row crosses shared memory twice
+// (written by the copy, read once) and is multiplied by packed FMAs (two columns an
+// instruction): at n = 128 a step takes about 1,250 cycles when its 64 KB are there,
+// against about 2,050 when the row was read again from shared memory for A^T r with
+// scalar FMAs, which held an iteration at 55.0 us whatever was prefetched (52.1 now;
+// bf16 hi + lo 70.1 -> 54.9, fp8 + bf16 61.2 -> 46.8, whose launches also had no
+// overlap with the u-solve and a separate reduction kernel; n = 96, m = 2765:
+// 25.0 -> 23.7).  The named barrier also frees the stage (every thread has its
+// columns in registers when it arrives), so no second mbarrier is needed.  RB rows
+// share one barrier where the columns per thread leave registers for them.
 #include <cuda_runtime.h>
+#include <cuda_fp8.h>
 
 #include "common.cuh"
 #include "kernels.h"
 
 namespace tvcs {
 
-constexpr int PROD_CONS = 512;           // 16 warps; thread 0 also issues the TMA copies
-constexpr int PROD_THREADS = PROD_CONS;
-constexpr int PROD_NST = 3;
 // Rows of A prefetched into L2 per block before the dependency wait, beyond the
 // ring: 1 MB (16 rows at n = 128; 136 blocks then hold about L2's capacity).
 constexpr size_t PROD_PF_BYTES = 1024 * 1024;
-// Bulk copies per stage of the ring.
-constexpr int PROD_TMA_PIECES = 1;
-// Stages ahead of each refill that are also prefetched into L2 while streaming
-// (0: only the pre-wait prefetch).
-constexpr int PROD_PF_STREAM = 0;
 
-template <int V, int RL, int RS>
+// TC column threads of V vectors of VW columns each (N = TC VW V), RL row lanes,
+// RB rows per lane and step; a stage of the ring holds one step's RL RB rows.
+template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
 struct ProdShape {
-    static constexpr int TPR = PROD_CONS / RL;
-    static constexpr int WPR = TPR / 32;
-    static constexpr int N = 4 * TPR * V;
-    static constexpr size_t STAGE_FLOATS = (size_t)RS * N;
-    static constexpr int YMAX = 1024;   // rows of y prefetched into shared memory
-    static constexpr size_t SMEM = PROD_NST * STAGE_FLOATS * 4 + 2 * PROD_NST * 8 +
-                                   2 * RL * WPR * 4 + 32 * 8 + 16 + YMAX * 4;
-    static_assert(RS % RL == 0, "rows per stage must be a multiple of the row lanes");
-    static_assert(TPR % 32 == 0, "row lanes must be whole warps");
+    static constexpr int THREADS = TC * RL, WARPS = THREADS / 32, WPR = TC / 32;
+    static constexpr int N = TC * VW * V, CPT = VW * V, RS = RL * RB;
+    static constexpr int B0 = PREC == 0 ? 4 : PREC == 1 ? 2 : 1, B1 = PREC == 0 ? 0 : 2;   // bytes per entry
+    static constexpr size_t P1_OFF = (size_t)RS * N * B0;          // second plane in a stage
+    static constexpr size_t STAGE = (size_t)RS * N * (B0 + B1);
+    static constexpr int YMAX = 1024;   // rows of y (and row scales) prefetched into shared memory
+    static constexpr size_t O_BAR = NST * STAGE;
+    static constexpr size_t O_RED = O_BAR + ((NST * 8 + 15) / 16) * 16;         // [2][RS][WPR]
+    static constexpr size_t O_DRED = O_RED + ((2 * RS * WPR * 4 + 15) / 16) * 16;   // [32] float2
+    static constexpr size_t O_FLAG = O_DRED + 32 * 8;
+    static constexpr size_t O_Y = O_FLAG + 16;
+    static constexpr size_t O_S = O_Y + YMAX * 4;
+    static constexpr size_t SMEM = O_S + (PREC == 2 ? YMAX * 4 : 0);
+    static_assert(TC % 32 == 0 && THREADS <= 512, "row lanes must be whole warps");
+    static_assert((N * B0) % 16 == 0, "TMA sizes are multiples of 16 bytes");
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+    static_assert(NST * STAGE >= (size_t)(RL - 1) * N * 4 && NST * STAGE >= (size_t)WARPS * 32 * 16,
+                  "the ring doubles as scratch of the epilogue");
 };
 
-// One block of 16 warps per SM (a three-stage ring of rows fills shared memory);
-// the grid leaves 16 SMs to the u-solve cluster of the same iteration, which
-// runs there while this kernel streams A.
-template <int V, int RL, int RS>
+namespace {
+
+__device__ __forceinline__ float lo16_f(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float hi16_f(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// BYTES of shared memory (4, 8 or 16, so aligned) as 32-bit words.
+template <int BYTES>
+__device__ __forceinline__ void lds_words(const unsigned char* p, uint32_t* w)
+{
+    static_assert(BYTES % 16 == 0 || BYTES == 8 || BYTES == 4 || BYTES == 2, "vector load");
+    if constexpr (BYTES % 16 == 0) {
+#pragma unroll
+        for (int k = 0; k < BYTES / 16; ++k) {
+            const uint4 v = reinterpret_cast<const uint4*>(p)[k];
+            w[4 * k] = v.x;
+            w[4 * k + 1] = v.y;
+            w[4 * k + 2] = v.z;
+            w[4 * k + 3] = v.w;
+        }
+    } else if constexpr (BYTES == 8) {
+        const uint2 v = *reinterpret_cast<const uint2*>(p);
+        w[0] = v.x;
+        w[1] = v.y;
+    } else if constexpr (BYTES == 4) {
+        w[0] = *reinterpret_cast<const uint32_t*>(p);
+    } else {
+        w[0] = *reinterpret_cast<const uint16_t*>(p);
+    }
+}
+
+// VW consecutive entries of one row, starting at column c, as packed pairs of
+// binary32: p0, p1 point at the row in the storage's planes, s is the row's scale (fp8).
+template <int PREC, int VW>
+__device__ __forceinline__ void load_entries(const unsigned char* p0, const unsigned char* p1, int c,
+                                             float s, uint64_t* a)
+{
+    if constexpr (PREC == 0) {
+        if constexpr (VW % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < VW / 4; ++k) {
+                const ulonglong2 v = reinterpret_cast<const ulonglong2*>(p0 + (size_t)c * 4)[k];
+                a[2 * k] = v.x;
+                a[2 * k + 1] = v.y;
+            }
+        } else {
+            a[0] = *reinterpret_cast<const uint64_t*>(p0 + (size_t)c * 4);
+        }
+    } else if constexpr (PREC == 1) {   // hi + lo, exact
+        uint32_t h[VW / 2], l[VW / 2];
+        lds_words<VW * 2>(p0 + (size_t)c * 2, h);
+        lds_words<VW * 2>(p1 + (size_t)c * 2, l);
+#pragma unroll
+        for (int k = 0; k < VW / 2; ++k)
+            a[k] = add2(pack2(lo16_f(h[k]), hi16_f(h[k])), pack2(lo16_f(l[k]), hi16_f(l[k])));
+    } else {   // s q + c, one rounding
+        uint32_t q[(VW + 3) / 4], cw[VW / 2];
+        lds_words<VW>(p0 + c, q);
+        lds_words<VW * 2>(p1 + (size_t)c * 2, cw);
+        const uint64_t s2 = pack2(s, s);
+#pragma unroll
+        for (int k = 0; k < VW / 2; ++k) {
+            const uint32_t pair = (q[k / 2] >> (16 * (k & 1))) & 0xffffu;
+            const float2 f = __half22float2(
+                __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)pair, __NV_E4M3)));
+            a[k] = fma2(s2, pack2(f.x, f.y), pack2(lo16_f(cw[k]), hi16_f(cw[k])));
+        }
+    }
+}
+
+}  // namespace
+
+// One block per SM (the ring fills shared memory at the larger sizes); the grid
+// leaves 16 SMs to the u-solve cluster of the same iteration, which runs there
+// while this kernel streams A.
+template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
 __global__ void __maxnreg__(128)
-    k_products(const float* __restrict__ A, int m, const float* __restrict__ x,
+    k_products(const unsigned char* __restrict__ P0, const unsigned char* __restrict__ P1,
+               const float* __restrict__ rscale, int m, const float* __restrict__ x,
                const float* __restrict__ y, float* __restrict__ r, float* __restrict__ gpart,
                float* __restrict__ g_out, float2* __restrict__ r2part, Ctrl* __restrict__ ctrl,
                int mode, cudaGraphConditionalHandle cond, int set_cond, long long budget, int pf,
                int bar_extra)
 {
-    using S = ProdShape<V, RL, RS>;
-    constexpr int N = S::N;
-    constexpr int TPR = S::TPR;
-    constexpr int WPR = S::WPR;
+    using S = ProdShape<PREC, TC, VW, V, RL, RB, NST>;
+    constexpr int N = S::N, WPR = S::WPR, RS = S::RS, CPT = S::CPT, THREADS = S::THREADS;
     extern __shared__ __align__(128) unsigned char smem[];
-    float* stage = reinterpret_cast<float*>(smem);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + PROD_NST * S::STAGE_FLOATS * 4);
-    uint64_t* empty = full + PROD_NST;
-    float* red = reinterpret_cast<float*>(empty + PROD_NST);        // [2][RL][WPR]
-    float2* dred = reinterpret_cast<float2*>(red + 2 * RL * WPR);   // [32]
-    int* sflag = reinterpret_cast<int*>(dred + 32);                 // [4]
-    float* sy = reinterpret_cast<float*>(sflag + 4);                // [YMAX]
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::O_BAR);
+    float* red = reinterpret_cast<float*>(smem + S::O_RED);
+    float2* dred = reinterpret_cast<float2*>(smem + S::O_DRED);
+    int* sflag = reinterpret_cast<int*>(smem + S::O_FLAG);
+    float* sy = reinterpret_cast<float*>(smem + S::O_Y);
+    float* ss = reinterpret_cast<float*>(smem + S::O_S);
 
     const int tid = threadIdx.x;
     const int G = gridDim.x;
@@ -82,36 +164,39 @@ __global__ void __maxnreg__(128)
     const int nst = (nrows + RS - 1) / RS;
 
     if (tid == 0) {
-        for (int s = 0; s < PROD_NST; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], PROD_CONS / 32);
-        }
+        for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
         fence_mbar_init();
     }
     __syncthreads();
 
     // The TMA copies are issued by thread 0.  A does not depend on the preceding
-    // kernel: the first PROD_NST stages go out before the dependency wait, so
+    // kernel: the first NST stages go out before the dependency wait, so
     // that under a programmatic dependent launch they stream in while the
     // u-solve still runs.
     const uint64_t pol = l2_policy_evict_first();
     auto issue = [&](int s) {
-        const int slot = s % PROD_NST;
-        const int rows = min(RS, nrows - s * RS);
-        const uint32_t bytes = (uint32_t)rows * N * 4u;
-        mbar_arrive_expect_tx(&full[slot], bytes);
-        tma_load_1d_split(stage + slot * S::STAGE_FLOATS, A + (size_t)(i0 + s * RS) * N, bytes,
-                          &full[slot], pol, PROD_TMA_PIECES);
+        const int slot = s % NST;
+        const int b0 = s * RS;
+        const size_t row = (size_t)(i0 + b0);
+        const uint32_t ent = (uint32_t)min(RS, nrows - b0) * N;
+        unsigned char* dst = smem + (size_t)slot * S::STAGE;
+        mbar_arrive_expect_tx(&full[slot], ent * (S::B0 + S::B1));
+        tma_load_1d(dst, P0 + row * N * S::B0, ent * S::B0, &full[slot], pol);
+        if constexpr (S::B1 > 0)
+            tma_load_1d(dst + S::P1_OFF, P1 + row * N * S::B1, ent * S::B1, &full[slot], pol);
     };
     // The pf stages after the ring are prefetched into L2 before the wait as
     // well (nothing waits for them): while the u-solve still runs, HBM streams
     // more of A than the ring holds, and the ring's later copies find those
     // rows in L2.  (Prefetching further ahead during the stream measured slower.)
     auto prefetch = [&](int s) {
-        const int rows = min(RS, nrows - s * RS);
-        prefetch_l2_bulk(A + (size_t)(i0 + s * RS) * N, (uint32_t)rows * N * 4u);
+        const int b0 = s * RS;
+        const size_t row = (size_t)(i0 + b0);
+        const uint32_t ent = (uint32_t)min(RS, nrows - b0) * N;
+        prefetch_l2_bulk(P0 + row * N * S::B0, ent * S::B0);
+        if constexpr (S::B1 > 0) prefetch_l2_bulk(P1 + row * N * S::B1, ent * S::B1);
     };
-    const int pre = min(PROD_NST, nst);
+    const int pre = min(NST, nst);
     int issued = 0;   // stages issued (thread 0)
     if (tid == 0) {
         for (; issued < pre; ++issued) issue(issued);
@@ -142,125 +227,166 @@ __global__ void __maxnreg__(128)
     }
 
     // ---------------- consumers ----------------
-    // y of this block's rows, prefetched so that r_i = dot - y_i waits on no global load.
-    const bool y_in_smem = (y != nullptr) && nrows <= S::YMAX;
-    if (y_in_smem)
-        for (int i = tid; i < nrows; i += PROD_CONS) sy[i] = y[i0 + i];
-    const int lane_row = tid / TPR;
-    const int ltid = tid - lane_row * TPR;
+    // y (and the scales) of this block's rows, prefetched so that no step waits on a
+    // global load for them.
+    const bool in_smem = nrows <= S::YMAX;
+    if (in_smem) {
+        for (int i = tid; i < nrows; i += THREADS) sy[i] = y != nullptr ? y[i0 + i] : 0.f;
+        if constexpr (PREC == 2)
+            for (int i = tid; i < nrows; i += THREADS) ss[i] = rscale[i0 + i];
+    }
+    const int lane_row = tid / TC;
+    const int ltid = tid - lane_row * TC;
     const int warp_in_row = ltid >> 5;
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    float4 xu[V], acc[V];
+    constexpr int CP = CPT / 2, VP = VW / 2;   // packed pairs of columns
+    uint64_t xu[CP], acc[CP];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        xu[v] = x4[ltid + v * TPR];
-        acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float* xv = x + (ltid + v * TC) * VW;
+        if constexpr (VW % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < VW / 4; ++k) {
+                const ulonglong2 t = reinterpret_cast<const ulonglong2*>(xv)[k];
+                xu[v * VP + 2 * k] = t.x;
+                xu[v * VP + 2 * k + 1] = t.y;
+            }
+        } else {
+            xu[v] = *reinterpret_cast<const uint64_t*>(xv);
+        }
     }
-    float2 r2 = make_float2(0.f, 0.f);   // double-single ||r||^2 of this thread's rows
+#pragma unroll
+    for (int c = 0; c < CP; ++c) acc[c] = 0ull;
+    named_barrier(1, THREADS);   // y and the scales are in shared memory
+    float2 r2 = make_float2(0.f, 0.f);   // double-single ||r||^2 of this lane's rows (ltid == 0)
     bool ok = true;
-    int step = 0;
+    // After a wait gave up, the steps go on with what is in shared memory (every thread
+    // stays with the block's barriers); the error word says that the results are void.
     for (int s = 0; s < nst; ++s) {
-        const int slot = s % PROD_NST;
-        if (ok && !mbar_wait(&full[slot], (s / PROD_NST) & 1, budget)) {
+        const int slot = s % NST;
+        if (ok && !mbar_wait(&full[slot], (s / NST) & 1, budget)) {
             set_error(ctrl, ERR_TIMEOUT);
             ok = false;
         }
-        const float* sb = stage + slot * S::STAGE_FLOATS;
-        const int rows = min(RS, nrows - s * RS);
-#pragma unroll 1
-        for (int st = 0; st < RS / RL; ++st, ++step) {
-            const int rl = st * RL + lane_row;
-            const bool valid = ok && rl < rows;
-            const float4* a4 = reinterpret_cast<const float4*>(sb + (size_t)rl * N);
-            const int li = s * RS + rl;   // row index within the block
-            float yi = 0.f;
-            if (valid && y != nullptr && !y_in_smem) yi = y[i0 + li];
-            float d = 0.f;
-            if (valid) {
+        const unsigned char* sb = smem + (size_t)slot * S::STAGE;
+        const int li0 = s * RS + lane_row * RB;   // first row of this lane's step, in the block
+        uint64_t a[RB][CP];
+        float* rb = red + ((s & 1) * RS + lane_row * RB) * WPR;
+        float d[RB];
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const float4 a = a4[ltid + v * TPR];
-                    d = fmaf(a.x, xu[v].x, d);
-                    d = fmaf(a.y, xu[v].y, d);
-                    d = fmaf(a.z, xu[v].z, d);
-                    d = fmaf(a.w, xu[v].w, d);
-                }
+        for (int b = 0; b < RB; ++b) {
+            if (RS == 1 || li0 + b < nrows) {
+                const size_t row = (size_t)(lane_row * RB + b) * N;
+                float sc = 1.f;
+                if constexpr (PREC == 2) sc = in_smem ? ss[li0 + b] : rscale[i0 + li0 + b];
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    load_entries<PREC, VW>(sb + row * S::B0, sb + S::P1_OFF + row * S::B1,
+                                           (ltid + v * TC) * VW, sc, &a[b][v * VP]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < CP; ++c) a[b][c] = 0ull;
             }
-            d = warp_sum(d);
-            float* rb = red + (step & 1) * RL * WPR;
-            if ((tid & 31) == 0) rb[lane_row * WPR + warp_in_row] = d;
-            named_barrier(1, PROD_CONS);
-            if (valid) {
-                float dot = 0.f;
+            uint64_t d0 = 0ull, d1 = 0ull;
 #pragma unroll
-                for (int w = 0; w < WPR; ++w) dot += rb[lane_row * WPR + w];
-                const int gi = i0 + li;
-                if (y_in_smem) yi = sy[li];
-                const float ri = dot - yi;
-                if (ltid == 0) {
-                    r[gi] = ri;
-                    r2 = ds_add(r2, ds_sq(ri));
-                }
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const float4 a = a4[ltid + v * TPR];
-                    acc[v].x = fmaf(ri, a.x, acc[v].x);
-                    acc[v].y = fmaf(ri, a.y, acc[v].y);
-                    acc[v].z = fmaf(ri, a.z, acc[v].z);
-                    acc[v].w = fmaf(ri, a.w, acc[v].w);
-                }
+            for (int c = 0; c < CP; ++c) {
+                if (c & 1)
+                    d1 = fma2(a[b][c], xu[c], d1);
+                else
+                    d0 = fma2(a[b][c], xu[c], d0);
             }
+            const float2 t = unpack2(add2(d0, d1));
+            d[b] = t.x + t.y;
         }
-        __syncwarp();
-        if ((tid & 31) == 0) mbar_arrive(&empty[slot]);
-        // refill this slot with stage s + PROD_NST once every warp is done with it
-        if (tid == 0 && s + PROD_NST < nst) {
-            if (ok && !mbar_wait(&empty[slot], (s / PROD_NST) & 1, budget)) {
-                set_error(ctrl, ERR_TIMEOUT);
-                ok = false;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int b = 0; b < RB; ++b) d[b] += __shfl_xor_sync(0xffffffffu, d[b], o);
+        if ((tid & 31) == 0) {
+#pragma unroll
+            for (int b = 0; b < RB; ++b) rb[b * WPR + warp_in_row] = d[b];
+        }
+        named_barrier(1, THREADS);   // the warps' parts are there, and nobody reads the stage any more
+        // refill this slot with stage s + NST
+        if (tid == 0 && ok && s + NST < nst) {
+            issue(s + NST);
+            ++issued;
+        }
+#pragma unroll
+        for (int b = 0; b < RB; ++b) {
+            const int li = li0 + b;
+            if (RS > 1 && li >= nrows) break;
+            float dot;
+            if constexpr (WPR % 4 == 0) {   // fixed tree over the warps' parts
+                uint64_t p[WPR / 2];
+#pragma unroll
+                for (int w = 0; w < WPR / 4; ++w) {
+                    const ulonglong2 t = reinterpret_cast<const ulonglong2*>(rb + b * WPR)[w];
+                    p[2 * w] = t.x;
+                    p[2 * w + 1] = t.y;
+                }
+#pragma unroll
+                for (int o = 1; o < WPR / 2; o *= 2)
+#pragma unroll
+                    for (int w = 0; w + o < WPR / 2; w += 2 * o) p[w] = add2(p[w], p[w + o]);
+                const float2 t = unpack2(p[0]);
+                dot = t.x + t.y;
+            } else {
+                dot = rb[b * WPR];
+#pragma unroll
+                for (int w = 1; w < WPR; ++w) dot += rb[b * WPR + w];
             }
-            if (ok) {
-                issue(s + PROD_NST);
-                ++issued;
-                // while streaming, prefetch into L2 the stage PROD_PF_STREAM stages past
-                // the one just issued
-                if (PROD_PF_STREAM > 0 && s + PROD_NST + PROD_PF_STREAM < nst)
-                    prefetch(s + PROD_NST + PROD_PF_STREAM);
+            const float ri = dot - (in_smem ? sy[li] : (y != nullptr ? y[i0 + li] : 0.f));
+            if (ltid == 0) {
+                r[i0 + li] = ri;
+                r2 = ds_add(r2, ds_sq(ri));
             }
+            const uint64_t rr = pack2(ri, ri);
+#pragma unroll
+            for (int c = 0; c < CP; ++c) acc[c] = fma2(rr, a[b][c], acc[c]);
         }
     }
     if (tid == 0 && !ok)   // a wait gave up: let the copies still in flight land (bounded)
-        for (int s = max(0, issued - PROD_NST); s < issued; ++s)
-            mbar_wait(&full[s % PROD_NST], (s / PROD_NST) & 1, drain_budget(budget));
+        for (int s = max(0, issued - NST); s < issued; ++s)
+            mbar_wait(&full[s % NST], (s / NST) & 1, drain_budget(budget));
 
     // ---------------- epilogue: partial A^T r and ||r||^2 ----------------
-    named_barrier(1, PROD_CONS);   // every consumer is done with the stage ring
-    float4* out4 = reinterpret_cast<float4*>(gpart + (size_t)blockIdx.x * N);
-    if constexpr (RL == 1) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) out4[ltid + v * TPR] = acc[v];
-    } else {
-        float4* scr = reinterpret_cast<float4*>(stage);   // (RL-1) x N/4 float4
+    named_barrier(1, THREADS);   // every consumer is done with the stage ring
+    float* out = gpart + (size_t)blockIdx.x * N;
+    float* scr = reinterpret_cast<float*>(smem);   // (RL-1) x N
+    if constexpr (RL > 1) {
         if (lane_row > 0) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) scr[(lane_row - 1) * (N / 4) + ltid + v * TPR] = acc[v];
+            for (int c = 0; c < CP; ++c)
+                *reinterpret_cast<uint64_t*>(scr + (size_t)(lane_row - 1) * N +
+                                             (ltid + (c / VP) * TC) * VW + 2 * (c % VP)) = acc[c];
         }
-        named_barrier(1, PROD_CONS);
+        named_barrier(1, THREADS);
         if (lane_row == 0) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                float4 t = acc[v];
-                for (int l = 1; l < RL; ++l) {
-                    const float4 o = scr[(l - 1) * (N / 4) + ltid + v * TPR];
-                    t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
-                }
-                out4[ltid + v * TPR] = t;
+            for (int c = 0; c < CP; ++c)
+                for (int l = 1; l < RL; ++l)
+                    acc[c] = add2(acc[c], *reinterpret_cast<const uint64_t*>(
+                                              scr + (size_t)(l - 1) * N + (ltid + (c / VP) * TC) * VW +
+                                              2 * (c % VP)));
+        }
+    }
+    if (lane_row == 0) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            float* ov = out + (ltid + v * TC) * VW;
+            if constexpr (VW % 4 == 0) {
+#pragma unroll
+                for (int k = 0; k < VW / 4; ++k)
+                    reinterpret_cast<ulonglong2*>(ov)[k] =
+                        make_ulonglong2(acc[v * VP + 2 * k], acc[v * VP + 2 * k + 1]);
+            } else {
+                *reinterpret_cast<uint64_t*>(ov) = acc[v];
             }
         }
     }
     // ||r||^2: one double-single value per row lane (held by ltid == 0)
     if (ltid == 0) dred[lane_row] = r2;
-    named_barrier(1, PROD_CONS);
+    named_barrier(1, THREADS);
     if (tid == 0) {
         float2 s = dred[0];
         for (int l = 1; l < RL; ++l) s = ds_add(s, dred[l]);
@@ -268,16 +394,16 @@ __global__ void __maxnreg__(128)
         // without the grid barrier below, the last block to arrive sums the partials
         sflag[0] = (g_out == nullptr && last_block_arrive(&ctrl->ticket_prod)) ? 1 : 0;
     }
-    named_barrier(1, PROD_CONS);
-    // ||r||^2 = sum of the G partials with all consumer warps (G <= 512), fixed order
+    named_barrier(1, THREADS);
+    // ||r||^2 = sum of the G partials with all warps (G <= THREADS), fixed order
     auto sum_r2 = [&]() {
         float2 v = tid < G ? __ldcg(r2part + tid) : make_float2(0.f, 0.f);
         v = warp_sum_ds(v);
         if ((tid & 31) == 0) dred[tid >> 5] = v;
-        named_barrier(1, PROD_CONS);
+        named_barrier(1, THREADS);
         if (tid == 0) {
             float2 t = dred[0];
-            for (int w = 1; w < PROD_CONS / 32; ++w) t = ds_add(t, dred[w]);
+            for (int w = 1; w < S::WARPS; ++w) t = ds_add(t, dred[w]);
             ctrl->r2 = ds_value(t);
         }
     };
@@ -287,7 +413,7 @@ __global__ void __maxnreg__(128)
     // ---------------- grid barrier, then g = sum of the G partials ----------------
     // All G blocks are co-resident (cooperative launch, one block per SM), so
     // a bounded spin on a monotone arrival counter is a grid barrier.
-    named_barrier(1, PROD_CONS);
+    named_barrier(1, THREADS);
     if (tid == 0) {
         __threadfence();
         const unsigned long long t = atomicAdd(&ctrl->gbar, 1ull);
@@ -304,19 +430,19 @@ __global__ void __maxnreg__(128)
         }
         __threadfence();
     }
-    named_barrier(1, PROD_CONS);
+    named_barrier(1, THREADS);
     if (blockIdx.x == 0) sum_r2();   // every block's partial is visible after the barrier
-    // This block's slice of float4 columns; warp w sums partials w, w+16, ... and
-    // warp 0 adds the 16 warp sums in order (deterministic).
+    // This block's slice of float4 columns; warp w sums partials w, w+WARPS, ... and
+    // warp 0 adds the warp sums in order (deterministic).
     const int N4 = N / 4;
     const int c0 = (int)(((long long)N4 * blockIdx.x) / G);
     const int c1 = (int)(((long long)N4 * (blockIdx.x + 1)) / G);
     const float4* gp4 = reinterpret_cast<const float4*>(gpart);
-    float4* sred = reinterpret_cast<float4*>(stage);   // [16][32], the stage ring is free
+    float4* sred = reinterpret_cast<float4*>(smem);   // [WARPS][32], the stage ring is free
     float4* g4 = reinterpret_cast<float4*>(g_out);
     const int lane = tid & 31, warp = tid >> 5;
-    constexpr int NWC = PROD_CONS / 32;   // consumer warps
-    constexpr int BATCH = 10;             // partials in flight per thread (G <= 160: one round)
+    constexpr int NWC = S::WARPS;
+    constexpr int BATCH = (160 + NWC - 1) / NWC;   // partials in flight per thread (G <= 160: one round)
     for (int base = c0; base < c1; base += 32) {
         const int c = base + lane;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -329,36 +455,37 @@ __global__ void __maxnreg__(128)
                     v[k] = p < G ? __ldcg(gp4 + (size_t)p * N4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
-                for (int k = 0; k < BATCH; ++k) {   // partials in increasing order, as before
+                for (int k = 0; k < BATCH; ++k) {   // partials in increasing order
                     s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w;
                 }
             }
         }
         sred[warp * 32 + lane] = s;
-        named_barrier(1, PROD_CONS);
+        named_barrier(1, THREADS);
         if (warp == 0 && c < c1) {
             float4 t = sred[lane];
 #pragma unroll
-            for (int w = 1; w < PROD_CONS / 32; ++w) {
+            for (int w = 1; w < NWC; ++w) {
                 const float4 v = sred[w * 32 + lane];
                 t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
             }
             g4[c] = t;
         }
-        named_barrier(1, PROD_CONS);
+        named_barrier(1, THREADS);
     }
 }
 
 // ---------------------------------------------------------------------------
-// Shape table: n -> (V, RL, RS).  N = n^2 = 4 * (512/RL) * V.
+// Shape table: (precision, n) -> (TC, VW, V, RL, RB, NST), and the rows a block
+// takes at least.  N = n^2 = TC VW V.
 // ---------------------------------------------------------------------------
-template <int V, int RL, int RS>
+template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
 static cudaError_t launch_prod_t(int grid, const ProdArgs& a, cudaStream_t s)
 {
-    using S = ProdShape<V, RL, RS>;
+    using S = ProdShape<PREC, TC, VW, V, RL, RB, NST>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(PROD_THREADS, 1, 1);
+    cfg.blockDim = dim3(S::THREADS, 1, 1);
     cfg.dynamicSmemBytes = S::SMEM;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -375,75 +502,73 @@ static cudaError_t launch_prod_t(int grid, const ProdArgs& a, cudaStream_t s)
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    const int pf = (int)(PROD_PF_BYTES / (S::STAGE_FLOATS * 4));
-    return cudaLaunchKernelEx(&cfg, k_products<V, RL, RS>, a.A, a.m, a.x, a.y, a.r, a.gpart,
-                              a.g_out, a.r2part, a.ctrl, a.mode,
+    const int pf = (int)(PROD_PF_BYTES / S::STAGE);
+    return cudaLaunchKernelEx(&cfg, k_products<PREC, TC, VW, V, RL, RB, NST>, a.P0, a.P1, a.rscale,
+                              a.m, a.x, a.y, a.r, a.gpart, a.g_out, a.r2part, a.ctrl, a.mode,
                               (cudaGraphConditionalHandle)a.cond, a.set_cond, a.budget, pf,
                               a.bar_extra);
 }
 
-template <int V, int RL, int RS>
+template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
 static cudaError_t configure_t()
 {
-    using S = ProdShape<V, RL, RS>;
-    return cudaFuncSetAttribute(k_products<V, RL, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)S::SMEM);
+    using S = ProdShape<PREC, TC, VW, V, RL, RB, NST>;
+    return cudaFuncSetAttribute(k_products<PREC, TC, VW, V, RL, RB, NST>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
 }
 
-#define TVCS_PROD_TABLE(X)   \
-    X(16, 1, 8, 64)          \
-    X(32, 2, 4, 16)          \
-    X(48, 9, 8, 8)           \
-    X(64, 4, 2, 4)           \
-    X(96, 9, 2, 2)           \
-    X(128, 8, 1, 1)
+//    precision, n, minimum rows per block, TC, VW, V, RL, RB, NST
+#define TVCS_PROD_TABLE(X)                \
+    X(0, 16, 8, 64, 4, 1, 8, 2, 4)        \
+    X(0, 32, 4, 256, 4, 1, 2, 4, 4)       \
+    X(0, 48, 4, 384, 2, 3, 1, 4, 4)       \
+    X(0, 64, 2, 512, 4, 2, 1, 4, 3)       \
+    X(0, 96, 1, 512, 2, 9, 1, 2, 3)       \
+    X(0, 128, 1, 512, 4, 8, 1, 1, 3)      \
+    X(1, 32, 4, 256, 4, 1, 2, 4, 4)       \
+    X(1, 64, 2, 512, 8, 1, 1, 4, 3)       \
+    X(1, 128, 1, 512, 8, 4, 1, 1, 3)      \
+    X(2, 32, 4, 256, 4, 1, 2, 4, 4)       \
+    X(2, 64, 2, 512, 8, 1, 1, 4, 4)       \
+    X(2, 128, 1, 512, 8, 4, 1, 1, 4)
 
-bool prod_supported(int n)
+bool prod_supported(int prec, int n)
 {
-    switch (n) {
-#define X(NN, V, RL, RS) case NN: return true;
-        TVCS_PROD_TABLE(X)
+#define X(PR, NN, MR, TC, VW, V, RL, RB, NST) \
+    if (prec == PR && n == NN) return true;
+    TVCS_PROD_TABLE(X)
 #undef X
-        default: return false;
-    }
+    return false;
 }
 
-static int prod_rl(int n)
+int prod_grid(int prec, int n, int m, int num_sms)
 {
-    switch (n) {
-#define X(NN, V, RL, RS) case NN: return RL;
-        TVCS_PROD_TABLE(X)
+    int mr = 1;
+#define X(PR, NN, MR, TC, VW, V, RL, RB, NST) \
+    if (prec == PR && n == NN) mr = MR;
+    TVCS_PROD_TABLE(X)
 #undef X
-        default: return 1;
-    }
-}
-
-int prod_grid(int n, int m, int num_sms)
-{
-    const int rl = prod_rl(n);
-    int g = (m + rl - 1) / rl;
+    const int g = (m + mr - 1) / mr;
     const int cap = num_sms > 32 ? num_sms - 16 : num_sms;   // 16 SMs stay free for the u-solve cluster
     return g < cap ? g : cap;
 }
 
-cudaError_t prod_configure(int n)
+cudaError_t prod_configure(int prec, int n)
 {
-    switch (n) {
-#define X(NN, V, RL, RS) case NN: return configure_t<V, RL, RS>();
-        TVCS_PROD_TABLE(X)
+#define X(PR, NN, MR, TC, VW, V, RL, RB, NST) \
+    if (prec == PR && n == NN) return configure_t<PR, TC, VW, V, RL, RB, NST>();
+    TVCS_PROD_TABLE(X)
 #undef X
-        default: return cudaErrorInvalidValue;
-    }
+    return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_products(int n, int grid, const ProdArgs& a, cudaStream_t s)
+cudaError_t launch_products(int prec, int n, int grid, const ProdArgs& a, cudaStream_t s)
 {
-    switch (n) {
-#define X(NN, V, RL, RS) case NN: return launch_prod_t<V, RL, RS>(grid, a, s);
-        TVCS_PROD_TABLE(X)
+#define X(PR, NN, MR, TC, VW, V, RL, RB, NST) \
+    if (prec == PR && n == NN) return launch_prod_t<PR, TC, VW, V, RL, RB, NST>(grid, a, s);
+    TVCS_PROD_TABLE(X)
 #undef X
-        default: return cudaErrorInvalidValue;
-    }
+    return cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------

@@ -1,6 +1,6 @@
-// Rows a6-a7 with A in reduced or split precision, and for images whose rows
-// are too long for one block: r = A x - y, partials of g = A^T r, one pass
-// over A (Xiao & Yang, eq. (line): g_k = A^T (A u^k - f)).
+// Rows a6-a7 for images whose rows are too long for one block (n = 192, 256; the
+// smaller ones: k_products.cu): r = A x - y, partials of g = A^T r, one pass over
+// A (Xiao & Yang, eq. (line): g_k = A^T (A u^k - f)), with A in any of its storages.
 //
 // Storage of A (m x N, row-major planes):
 //   FP32      one binary32 plane;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(CONS + 64, 1)
     int* sflag = reinterpret_cast<int*>(smem + S::O_S + QPROD_YMAX * 4);
 
     const int tid = threadIdx.x;
-    const uint32_t rank = CS > 1 ? cluster_rank() : 0u;
+    const uint32_t rank = cluster_rank();
     const int cidx = blockIdx.x / CS;          // cluster index = partial index
     const int G = gridDim.x / CS;              // number of clusters
     if (mode == MODE_ITER) {
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(CONS + 64, 1)
         fence_mbar_init();
     }
     __syncthreads();
-    if constexpr (CS > 1) cluster_sync_all();   // peers' barriers exist before any remote store
+    cluster_sync_all();   // peers' barriers exist before any remote store
 
     if (tid >= CONS + 32) {
         // ---------------- exchange warp: the block's part of every row to the cluster ----
@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(CONS + 64, 1)
         // block's own part of row s reached them, never overwrite a part that is still
         // to be read.
         const int lane = tid & 31;
-        const uint32_t xr = CS > 1 ? map_remote(smem_u32(xred), (uint32_t)(lane % CS)) : 0u;
-        const uint32_t xb = CS > 1 ? map_remote(smem_u32(xbar), (uint32_t)(lane % CS)) : 0u;
+        const uint32_t xr = map_remote(smem_u32(xred), (uint32_t)(lane % CS));
+        const uint32_t xb = map_remote(smem_u32(xbar), (uint32_t)(lane % CS));
         bool eok = true;
         for (int s = 0; s < nrows; ++s) {
             if (eok && !mbar_wait(&partbar[s & 1], (uint32_t)((s >> 1) & 1), budget)) {
@@ -198,16 +198,11 @@ __global__ void __launch_bounds__(CONS + 64, 1)
             float part = lane < WARPS ? red[(s & 1) * WARPS + lane] : 0.f;
             part = warp_sum(part);
             const int b = s & 3;
-            if constexpr (CS > 1) {
-                if (lane == 0) mbar_arrive_expect_tx(&xbar[b], (uint32_t)CS * 4u);
-                if (lane < CS) st_async_f32(xr + (uint32_t)((b * CS + rank) * 4), part, xb + (uint32_t)(b * 8));
-            } else if (lane == 0) {
-                xred[b] = part;
-                mbar_arrive(&xbar[b]);
-            }
+            if (lane == 0) mbar_arrive_expect_tx(&xbar[b], (uint32_t)CS * 4u);
+            if (lane < CS) st_async_f32(xr + (uint32_t)((b * CS + rank) * 4), part, xb + (uint32_t)(b * 8));
             __syncwarp();
         }
-        if constexpr (CS > 1) cluster_sync_all();
+        cluster_sync_all();
         return;
     }
     if (tid >= CONS) {
@@ -250,7 +245,7 @@ __global__ void __launch_bounds__(CONS + 64, 1)
         }
         __syncwarp();
         // stay for the final cluster barrier: no block leaves while peers may still write to it
-        if constexpr (CS > 1) cluster_sync_all();
+        cluster_sync_all();
         return;
     }
 
@@ -350,14 +345,11 @@ __global__ void __launch_bounds__(CONS + 64, 1)
         const int b = s & 3;
         const uint32_t phase = (uint32_t)((s >> 2) & 1);
         if (ok) {
-            bool got;
-            if constexpr (CS > 1) got = mbar_try_wait_cluster(&xbar[b], phase);
-            else got = mbar_try_wait(&xbar[b], phase);
+            bool got = mbar_try_wait_cluster(&xbar[b], phase);
             if (!got) {
                 const long long t0 = clock64();
                 for (;;) {
-                    if constexpr (CS > 1) got = mbar_try_wait_cluster(&xbar[b], phase);
-                    else got = mbar_try_wait(&xbar[b], phase);
+                    got = mbar_try_wait_cluster(&xbar[b], phase);
                     if (got) break;
                     if (clock64() - t0 > budget) {
                         set_error(ctrl, ERR_TIMEOUT);
@@ -448,7 +440,7 @@ __global__ void __launch_bounds__(CONS + 64, 1)
         }
     }
     __syncwarp();
-    if constexpr (CS > 1) {
+    {
         cluster_sync_all();
         // After a wait gave up, parts of the rows no longer awaited may still be on their
         // way into this block's shared memory (stores that complete on its barriers).
@@ -537,9 +529,7 @@ void launch_quant_fp8(const float* A, int m, int N, void* q, void* c, float* sca
 // ---------------------------------------------------------------------------
 #define TVCS_QPROD_TABLE(X)                                                              \
     X(0, 192, 9, 2, 512, 3) X(0, 256, 8, 4, 512, 3)                                      \
-    X(1, 32, 1, 1, 256, 3) X(1, 64, 2, 1, 512, 3) X(1, 128, 8, 1, 512, 3)                \
     X(1, 192, 9, 2, 512, 3) X(1, 256, 8, 4, 512, 3)                                      \
-    X(2, 32, 1, 1, 256, 4) X(2, 64, 2, 1, 512, 4) X(2, 128, 8, 1, 512, 4)                \
     X(2, 192, 9, 2, 512, 4) X(2, 256, 8, 4, 512, 4)
 
 template <int PREC, int V, int CS, int CONS, int NST>
@@ -557,12 +547,6 @@ static int qmax_clusters_t()
     if (qconfigure_t<PREC, V, CS, CONS, NST>() != cudaSuccess) {
         cudaGetLastError();
         return 0;
-    }
-    if (CS == 1) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        return sms;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CS, 1, 1);
@@ -599,7 +583,7 @@ static void qlaunch_t(int clusters, const QProdArgs& a, cudaStream_t s)
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = CS > 1 ? 1 : 0;
+    cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_products_q<PREC, V, CS, CONS, NST>, a.P0, a.P1, a.rscale, a.m, a.x,
                        a.y, a.r, a.gpart, a.r2part, a.ctrl, a.mode,
                        (cudaGraphConditionalHandle)a.cond, a.set_cond, a.budget);

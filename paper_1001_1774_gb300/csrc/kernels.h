@@ -64,9 +64,12 @@ void launch_usolve_img(int n, const TvArgs& a, cudaStream_t s);
 bool usolve_reg_configure();
 void launch_usolve_reg128(const TvArgs& a, cudaStream_t s);
 
-// Fused single-pass products r = A x - y, gpart = per-block partials of A^T r.
+// Fused single-pass products r = A x - y, gpart = per-block partials of A^T r, for
+// n <= 128 and every storage of A.
 struct ProdArgs {
-    const float* A;
+    const unsigned char* P0;  // binary32 plane | bf16 hi plane | e4m3 plane
+    const unsigned char* P1;  // unused | bf16 lo plane | bf16 correction plane
+    const float* rscale;      // per-row scale (fp8 storage), else unused
     int m;
     const float* x;
     const float* y;     // nullable
@@ -85,17 +88,17 @@ struct ProdArgs {
                         // raised by this many arrivals, which never come
 };
 
-bool prod_supported(int n);
-int prod_grid(int n, int m, int num_sms);   // number of blocks = number of partials P
-cudaError_t prod_configure(int n);          // opt-in shared memory size (call once per device)
+bool prod_supported(int prec, int n);
+int prod_grid(int prec, int n, int m, int num_sms);   // number of blocks = number of partials P
+cudaError_t prod_configure(int prec, int n);          // opt-in shared memory size (call once per device)
 // Both return the launch's own status.
-cudaError_t launch_products(int n, int grid, const ProdArgs& a, cudaStream_t s);
+cudaError_t launch_products(int prec, int n, int grid, const ProdArgs& a, cudaStream_t s);
 // g = sum_p gpart[p] (fixed order), wide grid; skipped when mode == MODE_ITER and ctrl->skip.
 cudaError_t launch_greduce(const float* gpart, int P, int N, float* g, const Ctrl* ctrl, int mode,
                            cudaStream_t s);
 
-// Products with A in binary32 (n = 192, 256), bf16 hi+lo, or fp8 e4m3 + bf16
-// correction: clusters of CS blocks split each row's columns.
+// The same products for n = 192 and 256 (binary32, bf16 hi+lo, or fp8 e4m3 + bf16
+// correction): clusters of CS blocks split each row's columns.
 struct QProdArgs {
     const unsigned char* P0;  // binary32 plane | bf16 hi plane | e4m3 plane
     const unsigned char* P1;  // unused | bf16 lo plane | bf16 correction plane

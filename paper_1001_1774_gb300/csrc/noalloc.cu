@@ -58,8 +58,8 @@ tvcs_status setup_device(int dev)
     if (e != cudaSuccess)
         return set_last_error(TVCS_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
     for (int n : {16, 32, 48, 64, 96, 128}) {
-        if (!prod_supported(n)) continue;
-        e = prod_configure(n);
+        if (!prod_supported(TVCS_PREC_FP32, n)) continue;
+        e = prod_configure(TVCS_PREC_FP32, n);
         if (e != cudaSuccess)
             return set_last_error(TVCS_ERR_CUDA, "configuring the product kernel: %s",
                                   cudaGetErrorString(e));
@@ -92,7 +92,7 @@ extern "C" tvcs_status tvcs_apply_noalloc(const float* A, int m, int n, const fl
         return set_last_error(TVCS_ERR_INVALID_ARG, "A, x, r and g must be non-NULL");
     if (m < 1 || m > (1 << 24))
         return set_last_error(TVCS_ERR_INVALID_ARG, "m = %d outside [1, 2^24]", m);
-    if (!prod_supported(n))
+    if (!prod_supported(TVCS_PREC_FP32, n))
         return set_last_error(TVCS_ERR_INVALID_ARG,
                               "n = %d not supported (16, 32, 48, 64, 96, 128)", n);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -124,7 +124,7 @@ extern "C" tvcs_status tvcs_apply_noalloc(const float* A, int m, int n, const fl
     if (st != TVCS_OK) return st;
 
     const int N = n * n;
-    const int P = prod_grid(n, m, g_num_sms[dev]);
+    const int P = prod_grid(TVCS_PREC_FP32, n, m, g_num_sms[dev]);
     const size_t b_gpart = round256((size_t)P * N * sizeof(float));
     const size_t b_r2 = round256((size_t)P * sizeof(float2));
     const size_t b_ctrl = round256(sizeof(Ctrl));
@@ -144,7 +144,7 @@ extern "C" tvcs_status tvcs_apply_noalloc(const float* A, int m, int n, const fl
     if (e != cudaSuccess)
         return set_last_error(TVCS_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     ProdArgs a{};
-    a.A = A;
+    a.P0 = reinterpret_cast<const unsigned char*>(A);
     a.m = m;
     a.x = x;
     a.y = y;
@@ -155,7 +155,7 @@ extern "C" tvcs_status tvcs_apply_noalloc(const float* A, int m, int n, const fl
     a.mode = MODE_PLAIN;
     a.budget = 1LL << 31;
     // Launch failures are this call's own: each launcher returns its launch status.
-    e = launch_products(n, P, a, s);
+    e = launch_products(TVCS_PREC_FP32, n, P, a, s);
     if (e == cudaSuccess) e = launch_greduce(gpart, P, N, g, ctrl, MODE_PLAIN, s);
     if (e != cudaSuccess) {
         cudaGetLastError();

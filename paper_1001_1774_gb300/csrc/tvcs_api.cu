@@ -12,6 +12,7 @@
 #include <new>
 #include <set>
 #include <string>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -53,7 +54,7 @@ tvcs_status fail(tvcs_status s, const char* fmt, ...)
     } while (0)
 
 std::mutex g_cfg_mutex;
-std::set<std::pair<int, int>> g_configured;  // (device, n) with the product kernel configured
+std::set<std::tuple<int, int, int>> g_configured;  // (device, precision, n) with the product kernel configured
 
 }  // namespace
 
@@ -132,7 +133,9 @@ void products(tvcs_ctx* h, const float* x, const float* y, float* r, float* gpar
         return;
     }
     ProdArgs a{};
-    a.A = h->A;
+    a.P0 = h->A ? reinterpret_cast<const unsigned char*>(h->A) : h->P0;
+    a.P1 = h->P1;
+    a.rscale = h->rscale;
     a.m = h->m;
     a.x = x;
     a.y = y;
@@ -147,7 +150,7 @@ void products(tvcs_ctx* h, const float* x, const float* y, float* r, float* gpar
     a.budget = budget_of(h);
     a.pdl = pdl;
     a.bar_extra = h->bar_extra;
-    launch_products(h->n, h->P, a, s);
+    launch_products(h->opt.precision, h->n, h->P, a, s);
 }
 
 // One iteration (rows a1-a7), MODE_ITER: the cluster u-solve, then the products
@@ -452,9 +455,10 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     CK(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->dev));
     {
         std::lock_guard<std::mutex> lk(g_cfg_mutex);
-        if (prod_supported(h->n) && !g_configured.count({h->dev, h->n})) {
-            CK(prod_configure(h->n));
-            g_configured.insert({h->dev, h->n});
+        const int prec = h->opt.precision;
+        if (prod_supported(prec, h->n) && !g_configured.count({h->dev, prec, h->n})) {
+            CK(prod_configure(prec, h->n));
+            g_configured.insert({h->dev, prec, h->n});
         }
     }
     if (h->opt.stream) {
@@ -471,7 +475,7 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     const bool regen = h->opt.a_mode == TVCS_A_REGENERATE;
     h->dct = dct_rows != nullptr;
     const bool noA = regen || h->dct;   // no stored matrix
-    h->use_q = !noA && !(prec == TVCS_PREC_FP32 && prod_supported(h->n));
+    h->use_q = !noA && !prod_supported(prec, h->n);
     if (noA) {
         h->P = 1;   // these products leave A^T r whole
     } else if (h->use_q) {
@@ -479,7 +483,7 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
         if (h->P == 0)
             return fail(TVCS_ERR_UNSUPPORTED, "no cluster of the product kernel fits (n = %d)", h->n);
     } else {
-        h->P = prod_grid(h->n, h->m, h->num_sms);
+        h->P = prod_grid(prec, h->n, h->m, h->num_sms);
     }
     h->ucluster = usolve_choose_cluster(h->n);
     if (h->ucluster == 0)
@@ -540,7 +544,7 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
         launch_gen_gauss(h->A, h->m, (int64_t)N, seed, scale, h->stream);
     }
     CKS(sync_and_check(h, "uploading A"));
-    if (h->use_q && !noA) {
+    if (!noA && (h->use_q || prec != TVCS_PREC_FP32)) {
         if (prec == TVCS_PREC_FP32) {
             h->P0 = reinterpret_cast<unsigned char*>(h->A);   // the plane is A itself
             h->A = nullptr;
@@ -583,8 +587,7 @@ tvcs_status copy_out(tvcs_ctx* h, float* dst, const float* src, size_t count)
 bool valid_n(int n, int prec)
 {
     if (!tv_supported(n)) return false;
-    if (prec == TVCS_PREC_FP32) return prod_supported(n) || qprod_supported(prec, n);
-    return qprod_supported(prec, n);
+    return prod_supported(prec, n) || qprod_supported(prec, n);
 }
 
 }  // namespace
@@ -987,7 +990,7 @@ tvcs_status tvcs_test_hold_grid_barrier(tvcs_handle h, int extra)
 {
     CKS(check_handle(h));
     if (extra < 0) return fail(TVCS_ERR_INVALID_ARG, "extra must be >= 0");
-    if (h->use_q || h->regen || h->dct)
+    if (h->use_q || h->regen || h->dct || h->opt.precision != TVCS_PREC_FP32)
         return fail(TVCS_ERR_UNSUPPORTED, "the hook acts on the binary32 product kernel (n <= 128)");
     if (h->bar_extra != extra) {
         h->bar_extra = extra;
