@@ -88,6 +88,11 @@ struct tvcs_ctx {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphExec_t tail[16] = {};
+    // the loop as one launch (n <= 96, stored A): blocks (0: the graphs above), exchange
+    // buffers, tags used so far
+    int loop_grid = 0;
+    uint64_t *ubuf = nullptr, *colx = nullptr, *rowx = nullptr, *nbuf = nullptr;
+    uint32_t loop_tag = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool state_ready = false;
     tvcs_batch* batch = nullptr;

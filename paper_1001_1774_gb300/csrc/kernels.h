@@ -97,6 +97,34 @@ cudaError_t launch_products(int prec, int n, int grid, const ProdArgs& a, cudaSt
 cudaError_t launch_greduce(const float* gpart, int P, int N, float* g, const Ctrl* ctrl, int mode,
                            cudaStream_t s);
 
+// The whole iteration loop of one problem with a stored A, n <= 96, as one cooperative
+// launch (k_loop.cu).  Buffers of tagged words (zeroed once): ubuf 2 N, colx and rowx
+// 2 n/2 n 2, nbuf 2 n/2 4.  Iteration k of a launch uses tag tag0 + k; tags never repeat.
+struct LoopArgs {
+    const unsigned char* P0;
+    const unsigned char* P1;
+    const float* rscale;
+    int m;
+    const float* y;           // data f
+    float *u, *w, *lam, *g, *r;   // the handle's state arrays
+    const float2* tw;
+    const float* s2;
+    float* gpart;             // grid x N
+    float2* r2part;           // grid
+    uint64_t *ubuf, *colx, *rowx, *nbuf;
+    Ctrl* ctrl;
+    float beta, mu_over_tau, mu;
+    int iters;                // >= 1
+    uint32_t tag0;
+    long long budget;         // spin-wait bound, SM cycles
+    int bar_extra;            // 0 outside the timeout test
+};
+// loop_configure: kernel attributes (once per device), false where the kernel cannot run;
+// loop_grid: blocks of the launch, 0 where the loop kernel does not apply.
+bool loop_configure(int prec, int n);
+int loop_grid(int prec, int n, int m, int num_sms);
+cudaError_t launch_loop(int prec, int n, int grid, const LoopArgs& a, cudaStream_t s);
+
 // The same products for n = 192 and 256 (binary32, bf16 hi+lo, or fp8 e4m3 + bf16
 // correction): clusters of CS blocks split each row's columns.
 struct QProdArgs {

@@ -55,6 +55,7 @@ tvcs_status fail(tvcs_status s, const char* fmt, ...)
 
 std::mutex g_cfg_mutex;
 std::set<std::tuple<int, int, int>> g_configured;  // (device, precision, n) with the product kernel configured
+std::set<std::tuple<int, int, int>> g_loop_configured;   // and the loop kernel
 
 }  // namespace
 
@@ -208,7 +209,7 @@ void free_ctx(tvcs_ctx* h)
     drop_loop_graphs(h);
     void* bufs[] = {h->A, h->f, h->u, h->w, h->lam, h->g, h->r, h->rhs, h->zeroN, h->tx, h->ty,
                     h->tr, h->tg, h->spec, h->tw, h->s2, h->gpart, h->gpart2, h->r2part, h->part,
-                    h->ctrl, h->P0, h->P1, h->rscale, h->dctC, h->dsidx, h->dsperm, h->drowptr};
+                    h->ctrl, h->P0, h->P1, h->rscale, h->ubuf, h->dctC, h->dsidx, h->dsperm, h->drowptr};
     for (void* p : bufs)
         if (p) cudaFree(p);
     if (h->hctrl) cudaFreeHost(h->hctrl);
@@ -331,18 +332,56 @@ tvcs_status init_state(tvcs_ctx* h, int init)
     return TVCS_OK;
 }
 
+// The loop as one launch (k_loop.cu).
+tvcs_status launch_iterations(tvcs_ctx* h, int iters)
+{
+    LoopArgs a{};
+    a.P0 = h->A ? reinterpret_cast<const unsigned char*>(h->A) : h->P0;
+    a.P1 = h->P1;
+    a.rscale = h->rscale;
+    a.m = h->m;
+    a.y = h->f;
+    a.u = h->u;
+    a.w = h->w;
+    a.lam = h->lam;
+    a.g = h->g;
+    a.r = h->r;
+    a.tw = h->tw;
+    a.s2 = h->s2;
+    a.gpart = h->gpart;
+    a.r2part = h->r2part;
+    a.ubuf = h->ubuf;
+    a.colx = h->colx;
+    a.rowx = h->rowx;
+    a.nbuf = h->nbuf;
+    a.ctrl = h->ctrl;
+    a.beta = (float)h->beta;
+    a.mu_over_tau = (float)(h->mu / h->tau);
+    a.mu = (float)h->mu;
+    a.iters = iters;
+    a.tag0 = h->loop_tag;
+    h->loop_tag += (uint32_t)iters;
+    a.budget = budget_of(h);
+    a.bar_extra = h->bar_extra;
+    CK(launch_loop(h->opt.precision, h->n, h->loop_grid, a, h->stream));
+    return TVCS_OK;
+}
+
 // Runs up to `iters` iterations from the current state; tol > 0 enables eq. (stop).
 tvcs_status run_loop(tvcs_ctx* h, int iters, double tol, tvcs_result* res)
 {
     // whole loop bodies in the WHILE graph, the remainder in a graph of its own
     const int nbody = iters / ITERS_PER_BODY, rest = iters % ITERS_PER_BODY;
-    if (!h->opt.host_loop) CKS(build_graph(h));
+    const bool one_launch = h->loop_grid > 0 && !h->opt.host_loop;
+    if (!h->opt.host_loop && !one_launch) CKS(build_graph(h));
     Ctrl& c = *h->hctrl;
     // loops_max: bodies of the WHILE graph (each ends by checking this bound)
     launch_run_begin(h->ctrl, iters, nbody, tol, h->opt.algo, h->stream);
     CK(cudaEventRecord(h->ev0, h->stream));
     if (iters > 0) {
-        if (h->opt.host_loop) {
+        if (one_launch) {
+            CKS(launch_iterations(h, iters));
+        } else if (h->opt.host_loop) {
             // Same kernels launched from the host, one iteration at a time (for
             // profilers that cannot look inside graphs with conditional nodes).
             for (int k = 0; k < iters; ++k) launch_iteration(h, 0ull, 0, h->stream, false);
@@ -453,13 +492,16 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
 {
     CK(cudaGetDevice(&h->dev));
     CK(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->dev));
+    bool loop_ok = false;
     {
         std::lock_guard<std::mutex> lk(g_cfg_mutex);
         const int prec = h->opt.precision;
         if (prod_supported(prec, h->n) && !g_configured.count({h->dev, prec, h->n})) {
             CK(prod_configure(prec, h->n));
             g_configured.insert({h->dev, prec, h->n});
+            if (loop_configure(prec, h->n)) g_loop_configured.insert({h->dev, prec, h->n});
         }
+        loop_ok = g_loop_configured.count({h->dev, prec, h->n}) != 0;
     }
     if (h->opt.stream) {
         h->stream = (cudaStream_t)h->opt.stream;
@@ -488,6 +530,8 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     h->ucluster = usolve_choose_cluster(h->n);
     if (h->ucluster == 0)
         return fail(TVCS_ERR_UNSUPPORTED, "no thread-block cluster of 8 or 16 fits for n = %d", h->n);
+    if (!noA && loop_ok) h->loop_grid = loop_grid(prec, h->n, h->m, h->num_sms);
+    const size_t P = (size_t)std::max(h->P, h->loop_grid);   // partials of A^T r
     const size_t nparts = 2 * (size_t)((N + 255) / 256 + 1024);
     // A: binary32 for the classic path and as the source of the split storages.
     if (!noA) CKS(alloc((void**)&h->A, sizeof(float) * m * N));
@@ -506,9 +550,18 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     CKS(alloc((void**)&h->spec, sizeof(float2) * (size_t)h->n * (h->n / 2 + 1)));
     CKS(alloc((void**)&h->tw, sizeof(float2) * (size_t)h->n));
     CKS(alloc((void**)&h->s2, sizeof(float) * (size_t)h->n));
-    CKS(alloc((void**)&h->gpart, sizeof(float) * N * (size_t)h->P));
+    CKS(alloc((void**)&h->gpart, sizeof(float) * N * P));
     CKS(alloc((void**)&h->gpart2, sizeof(float) * N * (size_t)h->P));
-    CKS(alloc((void**)&h->r2part, sizeof(float2) * (size_t)h->P));
+    CKS(alloc((void**)&h->r2part, sizeof(float2) * P));
+    if (h->loop_grid) {
+        // ubuf, colx, rowx of 2 N words and nbuf of 4 n, in one zeroed array
+        const size_t words = 6 * N + 4 * (size_t)h->n;
+        CKS(alloc((void**)&h->ubuf, sizeof(uint64_t) * words));
+        CK(cudaMemsetAsync(h->ubuf, 0, sizeof(uint64_t) * words, h->stream));
+        h->colx = h->ubuf + 2 * N;
+        h->rowx = h->colx + 2 * N;
+        h->nbuf = h->rowx + 2 * N;
+    }
     CKS(alloc((void**)&h->part, sizeof(double) * nparts));
     CKS(alloc((void**)&h->ctrl, sizeof(Ctrl)));
     CK(cudaMallocHost((void**)&h->hctrl, sizeof(Ctrl)));
