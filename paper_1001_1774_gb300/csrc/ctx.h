@@ -101,6 +101,8 @@ struct tvcs_ctx {
     bool dct = false;              // partial-DCT encoder (tvcs_create_partial_dct)
     float* dctC = nullptr;         // n x n DCT matrix, its transpose, 2 n x n scratch
     int *dsidx = nullptr, *dsperm = nullptr, *drowptr = nullptr;
+    int* dpos = nullptr;           // tables of its loop kernel (null: the graphs), k_dct_loop.cu
+    float2* dic = nullptr;
     tvcs_uneven* uneven = nullptr; // uneven batch whose first handle is this one
     int bar_extra = 0;             // timeout test hook (tvcs_test_hold_grid_barrier), else 0
     int gemm_force[4] = {0, 0, 0, 0};   // tvcs_test_gemm_shape: grid, pair of each batched GEMM (0: tuner)

@@ -213,4 +213,17 @@ __device__ __forceinline__ float2* fft_block(float2* a, float2* b, const float2*
     return FftRun<NN, INV, 0>::run(a, b, tw, nfft, dist, threadIdx.x, blockDim.x);
 }
 
+// FFT of one transform by one warp (buffers a and b in shared memory; returns the result's).
+template <int NN, bool INV, int S = 0>
+__device__ __forceinline__ float2* fft_warp(float2* a, float2* b, const float2* tw, int lane)
+{
+    if constexpr (S == fft_nstages(NN)) {
+        return a;
+    } else {
+        fft_stage<NN, S, INV>(a, b, tw, 1, NN, lane, 32);
+        __syncwarp();
+        return fft_warp<NN, INV, S + 1>(b, a, tw, lane);
+    }
+}
+
 }  // namespace tvcs

@@ -126,19 +126,6 @@ __device__ __forceinline__ ulonglong2 await2(const uint64_t* p, uint32_t tag, ul
     }
 }
 
-// FFT of one transform by one warp (buffers a and b in shared memory; returns the result's).
-template <int NN, bool INV, int S = 0>
-__device__ __forceinline__ float2* fft_warp(float2* a, float2* b, const float2* tw, int lane)
-{
-    if constexpr (S == fft_nstages(NN)) {
-        return a;
-    } else {
-        fft_stage<NN, S, INV>(a, b, tw, 1, NN, lane, 32);
-        __syncwarp();
-        return fft_warp<NN, INV, S + 1>(b, a, tw, lane);
-    }
-}
-
 template <int NN_, int PREC_, int TC_, int VW_, int V_, int RL_, int RB_, int RP_, int NPC_>
 struct LoopShape {
     using P = ProdShape<PREC_, TC_, VW_, V_, RL_, RB_, 2>;

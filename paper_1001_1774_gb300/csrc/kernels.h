@@ -265,6 +265,21 @@ bool dct_supported(int n);
 bool dct_configure(int n);   // kernel attributes (call once per device)
 void launch_dct_products(int n, const DctArgs& a, cudaStream_t s);
 
+// The whole iteration loop with the partial-DCT encoder as one cluster launch (k_dct_loop.cu).
+struct DctLoopArgs {
+    const float* y;           // data f
+    const int* pos;           // n x n by (k2, k1): place of coefficient k1 n + k2 in y and r, or -1
+    const float2* ic;         // s_k (cos, sin)(pi k / 2n), s_0 = 1/sqrt(n), else 1/sqrt(2n)
+    const float2* tw;
+    const float* s2;
+    float *u, *w, *lam, *g, *r;   // the handle's state arrays
+    Ctrl* ctrl;
+    float beta, mu_over_tau, mu;
+    int iters;                // >= 1
+};
+bool dct_loop_configure(int n);   // kernel attributes; false where the kernel cannot run
+cudaError_t launch_dct_loop(int n, const DctLoopArgs& a, cudaStream_t s);
+
 // Loop condition of a batch: continue while any of ctrls[0..count) runs and
 // bctrl->loops stays below bctrl->loops_max (batch.cu).
 // With slot_img / img_slot set (count <= 512), also packs the running images

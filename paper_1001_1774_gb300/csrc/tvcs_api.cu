@@ -209,7 +209,8 @@ void free_ctx(tvcs_ctx* h)
     drop_loop_graphs(h);
     void* bufs[] = {h->A, h->f, h->u, h->w, h->lam, h->g, h->r, h->rhs, h->zeroN, h->tx, h->ty,
                     h->tr, h->tg, h->spec, h->tw, h->s2, h->gpart, h->gpart2, h->r2part, h->part,
-                    h->ctrl, h->P0, h->P1, h->rscale, h->ubuf, h->dctC, h->dsidx, h->dsperm, h->drowptr};
+                    h->ctrl, h->P0, h->P1, h->rscale, h->ubuf, h->dctC, h->dsidx, h->dsperm, h->drowptr,
+                    h->dpos, h->dic};
     for (void* p : bufs)
         if (p) cudaFree(p);
     if (h->hctrl) cudaFreeHost(h->hctrl);
@@ -332,9 +333,29 @@ tvcs_status init_state(tvcs_ctx* h, int init)
     return TVCS_OK;
 }
 
-// The loop as one launch (k_loop.cu).
+// The loop as one launch (k_loop.cu, k_dct_loop.cu).
 tvcs_status launch_iterations(tvcs_ctx* h, int iters)
 {
+    if (h->dct) {
+        DctLoopArgs d{};
+        d.y = h->f;
+        d.pos = h->dpos;
+        d.ic = h->dic;
+        d.tw = h->tw;
+        d.s2 = h->s2;
+        d.u = h->u;
+        d.w = h->w;
+        d.lam = h->lam;
+        d.g = h->g;
+        d.r = h->r;
+        d.ctrl = h->ctrl;
+        d.beta = (float)h->beta;
+        d.mu_over_tau = (float)(h->mu / h->tau);
+        d.mu = (float)h->mu;
+        d.iters = iters;
+        CK(launch_dct_loop(h->n, d, h->stream));
+        return TVCS_OK;
+    }
     LoopArgs a{};
     a.P0 = h->A ? reinterpret_cast<const unsigned char*>(h->A) : h->P0;
     a.P1 = h->P1;
@@ -372,7 +393,7 @@ tvcs_status run_loop(tvcs_ctx* h, int iters, double tol, tvcs_result* res)
 {
     // whole loop bodies in the WHILE graph, the remainder in a graph of its own
     const int nbody = iters / ITERS_PER_BODY, rest = iters % ITERS_PER_BODY;
-    const bool one_launch = h->loop_grid > 0 && !h->opt.host_loop;
+    const bool one_launch = (h->loop_grid > 0 || h->dpos) && !h->opt.host_loop;
     if (!h->opt.host_loop && !one_launch) CKS(build_graph(h));
     Ctrl& c = *h->hctrl;
     // loops_max: bodies of the WHILE graph (each ends by checking this bound)
@@ -485,6 +506,19 @@ tvcs_status dct_init(tvcs_ctx* h, const int32_t* rows)
     CK(cudaMemcpy(h->dsidx, sidx.data(), sizeof(int) * (size_t)m, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->dsperm, sperm.data(), sizeof(int) * (size_t)m, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->drowptr, rowptr.data(), sizeof(int) * (size_t)(n + 1), cudaMemcpyHostToDevice));
+    if (dct_loop_configure(n)) {
+        std::vector<int> pos((size_t)n * n, -1);
+        for (int i = 0; i < m; ++i) pos[(size_t)(rows[i] % n) * n + rows[i] / n] = i;
+        std::vector<float2> ic(n);
+        for (int k = 0; k < n; ++k) {
+            const double s = k == 0 ? sqrt(1.0 / n) : sqrt(0.5 / n);
+            ic[k] = make_float2((float)(s * cos(pi * k / (2.0 * n))), (float)(s * sin(pi * k / (2.0 * n))));
+        }
+        CKS(alloc((void**)&h->dpos, sizeof(int) * pos.size()));
+        CKS(alloc((void**)&h->dic, sizeof(float2) * (size_t)n));
+        CK(cudaMemcpy(h->dpos, pos.data(), sizeof(int) * pos.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(h->dic, ic.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice));
+    }
     return TVCS_OK;
 }
 

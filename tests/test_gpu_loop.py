@@ -90,3 +90,34 @@ def test_loop_stops_by_the_relative_change(tv, n, mu, beta, tol):
     res = tv.tvcs_solve(h, P.f, u)
     assert res.stopped_by_tol == ref.info["stopped_by_tol"] and abs(res.iters - ref.info["iters"]) <= 1
     assert rel(u, ref.u) <= (tol if res.stopped_by_tol else 1e-4)   # one iteration more or less moves u by tol
+
+
+# The partial-DCT encoder's loop (one cluster): every side, one / few / all coefficients in a
+# shuffled order, both algorithms, one iteration, a run in parts, a stop by eq. (stop).
+@pytest.mark.parametrize("n,m,algo,iters,tol", [
+    (16, 76, 0, 20, 0.0), (16, 256, 1, 1, 0.0), (32, 1, 0, 10, 0.0), (32, 511, 1, 30, 0.0), (48, 461, 0, 25, 0.0),
+    (64, 2049, 0, 40, 0.0), (96, 921, 1, 17, 0.0), (96, 9216, 0, 8, 0.0), (128, 4915, 0, 40, 0.0),
+    (128, 4915, 0, 400, 3e-3), (128, 16383, 0, 5, 0.0)])
+def test_dct_loop_against_the_oracle_and_the_single_launches(tv, n, m, algo, iters, tol):
+    rng = np.random.default_rng(n + m)
+    rows = rng.choice(n * n, size=m, replace=False).astype(np.int32)
+    f = synth.measure_dct(rows, synth.phantom(n, 8, 5), 1e-3, 77)
+    ref = oracle.solve_dct(rows, f, n, 500.0, 64.0, 1.9, tol=tol, max_iter=iters, algo=algo)
+    out = []
+    for host_loop in (0, 1):
+        opt = tv.tvcs_default_options()
+        opt.tau, opt.max_iter, opt.algo, opt.host_loop = 1.9, iters, algo, host_loop
+        h = tv.tvcs_create_partial_dct(rows, n, 500.0, 64.0, tol, opt)
+        u = np.empty(n * n, np.float32)
+        res = tv.tvcs_solve(h, f, u)
+        assert res.stopped_by_tol == ref.info["stopped_by_tol"] and abs(res.iters - ref.info["iters"]) <= 1
+        assert rel(u, ref.u) <= (1e-5 if tol == 0.0 else tol)
+        r = tv.get_state(h, tv.TVCS_STATE_R).astype(np.float64)
+        assert abs(res.resid2 - (r * r).sum()) <= 1e-9 * res.resid2
+        tv.tvcs_iterate(h, 3)
+        tv.tvcs_iterate(h, 1)
+        out.append([tv.get_state(h, k) for k in (tv.TVCS_STATE_U, tv.TVCS_STATE_W, tv.TVCS_STATE_LAMBDA)])
+        tv.tvcs_destroy(h)
+    if tol == 0.0:
+        for a, b in zip(*out):
+            assert rel(a, b) <= 3e-5 or np.linalg.norm(b) == 0.0
