@@ -21,7 +21,9 @@
  * Conventions for every entry point:
  *  - Pointers to arrays may be host (pageable or pinned) or device pointers;
  *    the library detects the kind with cudaPointerGetAttributes and copies
- *    through its own device buffers.  The caller keeps ownership of every
+ *    through its own device buffers (tvcs_apply reads and writes arrays in the
+ *    handle's device memory in place where their alignment allows it and no
+ *    result overlaps another array).  The caller keeps ownership of every
  *    array it passes; the library keeps no pointer to caller memory after a
  *    call returns.
  *  - All device work is ordered on the handle's stream (tvcs_options.stream).
@@ -312,7 +314,8 @@ tvcs_status tvcs_test_gemm_shape(tvcs_handle h, int grid1, int pair1, int grid2,
  * until the process exits.  Sizes whose partial sums do not fit return
  * TVCS_ERR_INVALID_ARG with a message naming the limit.  The first call on a
  * device performs one-time set-up on that device (it looks up the array's
- * device address and sets the kernels' shared-memory limit).  Every call on a
+ * device address, sets the kernels' shared-memory limit and, once per process,
+ * page-locks one page of the library's own host memory for a status word).  Every call on a
  * device shares the same array and clears the parts that must start at zero,
  * so calls whose device work overlaps (other host threads, other streams)
  * race on it and must be serialised by the caller. */

@@ -114,20 +114,22 @@ def _check(status: int) -> int:
     return status
 
 
+try:
+    import torch as _torch
+except ImportError:   # numpy arrays only
+    _torch = None
+
+
 def _ptr(x, count: int | None = None, writable: bool = False):
     """Raw pointer of a contiguous float32 torch tensor or numpy array (host or device)."""
     if x is None:
         return None
-    try:
-        import torch
-        if isinstance(x, torch.Tensor):
-            if x.dtype != torch.float32 or not x.is_contiguous():
-                raise TypeError("expected a contiguous float32 tensor")
-            if count is not None and x.numel() != count:
-                raise ValueError("expected %d elements, got %d" % (count, x.numel()))
-            return ctypes.c_void_p(x.data_ptr())
-    except ImportError:
-        pass
+    if _torch is not None and isinstance(x, _torch.Tensor):
+        if x.dtype != _torch.float32 or not x.is_contiguous():
+            raise TypeError("expected a contiguous float32 tensor")
+        if count is not None and x.numel() != count:
+            raise ValueError("expected %d elements, got %d" % (count, x.numel()))
+        return ctypes.c_void_p(x.data_ptr())
     if isinstance(x, np.ndarray):
         if x.dtype != np.float32 or not x.flags.c_contiguous:
             raise TypeError("expected a C-contiguous float32 array")
@@ -144,17 +146,15 @@ def _ready(*arrays) -> None:
     wait for other streams.  Before a call that reads or writes torch CUDA tensors,
     finish the work queued on torch's current stream of each device involved (the
     tensors' producers, and pending readers of output buffers): once per device."""
-    try:
-        import torch
-    except ImportError:
+    if _torch is None:
         return
     devs = set()
     for a in arrays:
         for x in (a if isinstance(a, (list, tuple)) else (a,)):
-            if isinstance(x, torch.Tensor) and x.is_cuda:
-                devs.add(x.device)
+            if isinstance(x, _torch.Tensor) and x.is_cuda:
+                devs.add(x.get_device())
     for d in devs:
-        torch.cuda.current_stream(d).synchronize()
+        _torch.cuda.current_stream(d).synchronize()
 
 
 def tvcs_default_options() -> tvcs_options:

@@ -62,6 +62,17 @@ __device__ __forceinline__ void set_error(Ctrl* c, int code)
     atomicCAS(&c->error, ERR_NONE, code);
 }
 
+// The same, and into the host's word where the caller passed one (pinned memory that the
+// host reads after the stream has finished: a call that succeeds copies nothing back).
+__device__ __forceinline__ void set_error(Ctrl* c, int code, int* host_word)
+{
+    set_error(c, code);
+    if (host_word) {
+        *reinterpret_cast<volatile int*>(host_word) = code;
+        __threadfence_system();
+    }
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

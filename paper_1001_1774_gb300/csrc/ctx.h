@@ -83,6 +83,7 @@ struct tvcs_ctx {
     double* part = nullptr;
     tvcs::Ctrl* ctrl = nullptr;
     tvcs::Ctrl* hctrl = nullptr;  // pinned host mirror
+    int* herr = nullptr;          // pinned word after it: timeouts of tvcs_apply's products
     // loop graph (a WHILE node over bodies of 16 iterations) and the graphs of
     // 1..15 iterations that end a run whose length is not a multiple of 16
     cudaGraph_t graph = nullptr;

@@ -49,7 +49,7 @@ __global__ void __maxnreg__(128)
                const float* __restrict__ y, float* __restrict__ r, float* __restrict__ gpart,
                float* __restrict__ g_out, float2* __restrict__ r2part, Ctrl* __restrict__ ctrl,
                int mode, cudaGraphConditionalHandle cond, int set_cond, long long budget, int pf,
-               int bar_extra)
+               int bar_extra, int* host_err)
 {
     using S = ProdShape<PREC, TC, VW, V, RL, RB, NST>;
     constexpr int N = S::N, WPR = S::WPR, RS = S::RS, CPT = S::CPT, THREADS = S::THREADS;
@@ -169,7 +169,7 @@ __global__ void __maxnreg__(128)
     for (int s = 0; s < nst; ++s) {
         const int slot = s % NST;
         if (ok && !mbar_wait(&full[slot], (s / NST) & 1, budget)) {
-            set_error(ctrl, ERR_TIMEOUT);
+            set_error(ctrl, ERR_TIMEOUT, host_err);
             ok = false;
         }
         const unsigned char* sb = smem + (size_t)slot * S::STAGE;
@@ -329,7 +329,7 @@ __global__ void __maxnreg__(128)
         const long long t0 = clock64();
         while (ld_acquire_u64(&ctrl->gbar) < target) {
             if (clock64() - t0 > budget) {
-                set_error(ctrl, ERR_TIMEOUT);
+                set_error(ctrl, ERR_TIMEOUT, host_err);
                 break;
             }
         }
@@ -411,7 +411,7 @@ static cudaError_t launch_prod_t(int grid, const ProdArgs& a, cudaStream_t s)
     return cudaLaunchKernelEx(&cfg, k_products<PREC, TC, VW, V, RL, RB, NST>, a.P0, a.P1, a.rscale,
                               a.m, a.x, a.y, a.r, a.gpart, a.g_out, a.r2part, a.ctrl, a.mode,
                               (cudaGraphConditionalHandle)a.cond, a.set_cond, a.budget, pf,
-                              a.bar_extra);
+                              a.bar_extra, a.host_err);
 }
 
 template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
@@ -581,6 +581,30 @@ __global__ void k_run_begin(Ctrl* __restrict__ c, int max_iter, int loops_max, d
     c->algo = algo;
     c->lbar = 0ull;
     c->ticket_fft = c->ticket_prod = c->ticket_fin = c->ticket_w = c->ticket_gather = 0u;
+}
+
+// Start point of a solve, on the device (no host round trip).
+__global__ void k_init_state(Ctrl* __restrict__ c, float* __restrict__ w, float* __restrict__ lam, int N,
+                             int given)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (given) {   // w^0 = 0 in the current copy; u and lambda are the caller's
+        const int par = c->wpar;
+        if (i < 2 * N) w[(size_t)par * 2 * N + i] = 0.f;
+    } else if (i < 4 * N) {
+        w[i] = 0.f;
+        lam[i] = 0.f;
+    }
+    if (i == 0) {
+        c->pending = 0;
+        if (!given) c->wpar = 0;
+        c->error = 0;
+    }
+}
+
+void launch_init_state(Ctrl* c, float* w, float* lam, int N, int given, cudaStream_t s)
+{
+    k_init_state<<<(4 * N + 255) / 256, 256, 0, s>>>(c, w, lam, N, given);
 }
 
 void launch_run_begin(Ctrl* c, int max_iter, int loops_max, double tol, int algo, cudaStream_t s)

@@ -86,6 +86,7 @@ struct ProdArgs {
     int pdl;            // launch with a programmatic dependency on the preceding grid
     int bar_extra;      // 0; > 0 only in the timeout test: the grid barrier's target is
                         // raised by this many arrivals, which never come
+    int* host_err;      // nullable: pinned host word that receives a timeout as well
 };
 
 bool prod_supported(int prec, int n);
@@ -296,6 +297,9 @@ void launch_gather(const float* gpart, int P, int N, float scale, float* out, do
 // v = z / sqrt(ctrl->vec2)
 void launch_normalize(const float* z, float* v, int N, const Ctrl* ctrl, cudaStream_t s);
 void launch_fill(float* v, int N, float value, cudaStream_t s);
+// Start point of a solve: pending = 0, error = 0, then wpar = 0 and w = lambda = 0 (given = 0),
+// or w^0 = 0 in the current copy (given = 1).  N pixels.
+void launch_init_state(Ctrl* c, float* w, float* lam, int N, int given, cudaStream_t s);
 // it, max_iter, done, skip, stop_by_tol, loops, loops_max, tol, error, algo and the
 // tickets of a control block for a new run
 void launch_run_begin(Ctrl* c, int max_iter, int loops_max, double tol, int algo, cudaStream_t s);

@@ -35,8 +35,16 @@ constexpr int kMaxDevices = 64;
 // double-single partials of ||r||^2 and a control block for the last-block ticket.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
+// One host word per device, on a page of its own that the one-time set-up page-locks: the
+// kernels record a bounded wait that gave up there, so that a call copies nothing back (a
+// 4-byte copy to pageable memory took about 15 us of a call's 54).
+alignas(4096) int g_err_word[4096 / sizeof(int)];
+static_assert(kMaxDevices <= 4096 / (int)sizeof(int), "one word per device");
+bool g_err_page_tried = false, g_err_page_locked = false;
+
 std::mutex g_setup_mutex;
 void* g_scratch_ptr[kMaxDevices] = {};
+int* g_err_dev[kMaxDevices] = {};   // device address of the word; null: the word is copied back
 int g_num_sms[kMaxDevices] = {};
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -64,6 +72,20 @@ tvcs_status setup_device(int dev)
             return set_last_error(TVCS_ERR_CUDA, "configuring the product kernel: %s",
                                   cudaGetErrorString(e));
     }
+    // (in relaxed capture mode, so that a capture of another thread is not disturbed)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess) {
+        if (!g_err_page_tried) {
+            g_err_page_tried = true;
+            g_err_page_locked = cudaHostRegister(g_err_word, sizeof(g_err_word),
+                                                 cudaHostRegisterPortable | cudaHostRegisterMapped) == cudaSuccess;
+        }
+        void* d = nullptr;
+        if (g_err_page_locked && cudaHostGetDevicePointer(&d, &g_err_word[dev], 0) == cudaSuccess)
+            g_err_dev[dev] = static_cast<int*>(d);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    cudaGetLastError();   // without the page the error word is copied back
     g_num_sms[dev] = sms;
     g_scratch_ptr[dev] = p;
     return TVCS_OK;
@@ -154,19 +176,31 @@ extern "C" tvcs_status tvcs_apply_noalloc(const float* A, int m, int n, const fl
     a.ctrl = ctrl;
     a.mode = MODE_PLAIN;
     a.budget = 1LL << 31;
+    a.host_err = g_err_dev[dev];
+    volatile int* word = &g_err_word[dev];
+    *word = ERR_NONE;
+    // One launch that reduces its partials behind a grid barrier; where its blocks cannot all be
+    // resident (a context with fewer SMs), the partials are reduced by a second launch.
     // Launch failures are this call's own: each launcher returns its launch status.
+    a.g_out = g;
     e = launch_products(TVCS_PREC_FP32, n, P, a, s);
-    if (e == cudaSuccess) e = launch_greduce(gpart, P, N, g, ctrl, MODE_PLAIN, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        a.g_out = nullptr;
+        e = launch_products(TVCS_PREC_FP32, n, P, a, s);
+        if (e == cudaSuccess) e = launch_greduce(gpart, P, N, g, ctrl, MODE_PLAIN, s);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_last_error(TVCS_ERR_CUDA, "tvcs_apply_noalloc: launch failed: %s",
                               cudaGetErrorString(e));
     }
-    int err_word = 0;
-    e = cudaMemcpyAsync(&err_word, &ctrl->error, sizeof(int), cudaMemcpyDeviceToHost, s);
+    int err_word = ERR_NONE;
+    if (!g_err_dev[dev]) e = cudaMemcpyAsync(&err_word, &ctrl->error, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess)
         return set_last_error(TVCS_ERR_CUDA, "tvcs_apply_noalloc: %s", cudaGetErrorString(e));
+    if (g_err_dev[dev]) err_word = *word;
     if (err_word == ERR_TIMEOUT)
         return set_last_error(TVCS_ERR_TIMEOUT, "a bounded device wait gave up");
     return TVCS_OK;

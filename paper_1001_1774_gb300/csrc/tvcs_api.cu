@@ -88,7 +88,8 @@ TvArgs tv_args(tvcs_ctx* h, int mode, bool stage_outputs)
 
 // r = A x - y and the partials of A^T r into gpart; then g = their sum when g != NULL.
 void products(tvcs_ctx* h, const float* x, const float* y, float* r, float* gpart, float* g,
-              int mode, unsigned long long cond, int set_cond, cudaStream_t s, int pdl = 0)
+              int mode, unsigned long long cond, int set_cond, cudaStream_t s, int pdl = 0,
+              int* host_err = nullptr)
 {
     if (h->regen) {   // A regenerated in the kernel; A^T r whole in g, else in gpart (P = 1)
         regen_products(h, x, y, r, g ? g : gpart, mode, cond, set_cond, s);
@@ -151,6 +152,7 @@ void products(tvcs_ctx* h, const float* x, const float* y, float* r, float* gpar
     a.budget = budget_of(h);
     a.pdl = pdl;
     a.bar_extra = h->bar_extra;
+    a.host_err = host_err;
     launch_products(h->opt.precision, h->n, h->P, a, s);
 }
 
@@ -302,33 +304,22 @@ void refresh_products(tvcs_ctx* h)
 
 tvcs_status init_state(tvcs_ctx* h, int init)
 {
-    const size_t N = (size_t)h->N;
     if (init == TVCS_INIT_GIVEN) {
         // Warm start: keep the caller's u and lambda (tvcs_set_state), w^0 = 0.
         if (!h->state_ready) return fail(TVCS_ERR_INVALID_ARG, "INIT_GIVEN needs tvcs_set_state(U) first");
         refresh_products(h);
-        CKS(read_ctrl(h));   // after the kernels: the host copy is current
-        const int par = h->hctrl->wpar;
-        CK(cudaMemsetAsync(h->w + (size_t)par * 2 * N, 0, sizeof(float) * 2 * N, h->stream));
-        h->hctrl->pending = 0;
-        h->hctrl->error = 0;
-        return write_ctrl(h);
+        launch_init_state(h->ctrl, h->w, h->lam, h->N, 1, h->stream);
+        return TVCS_OK;
     }
-    CK(cudaMemsetAsync(h->w, 0, sizeof(float) * 4 * N, h->stream));
-    CK(cudaMemsetAsync(h->lam, 0, sizeof(float) * 4 * N, h->stream));
     if (init == TVCS_INIT_ATF) {
         // u^0 = A^T f (reading C3): the products at x = 0 give A^T (0 - f).
         products(h, h->zeroN, h->f, h->r, h->gpart, nullptr, MODE_PLAIN, 0ull, 0, h->stream);
         launch_gather(h->gpart, h->P, h->N, -1.0f, h->u, h->part, h->ctrl, h->stream);
     } else if (init == TVCS_INIT_ZERO) {
-        CK(cudaMemsetAsync(h->u, 0, sizeof(float) * N, h->stream));
+        CK(cudaMemsetAsync(h->u, 0, sizeof(float) * (size_t)h->N, h->stream));
     }
     refresh_products(h);
-    CKS(read_ctrl(h));
-    h->hctrl->pending = 0;
-    h->hctrl->wpar = 0;
-    h->hctrl->error = 0;
-    CKS(write_ctrl(h));
+    launch_init_state(h->ctrl, h->w, h->lam, h->N, 0, h->stream);
     h->state_ready = true;
     return TVCS_OK;
 }
@@ -598,8 +589,9 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     }
     CKS(alloc((void**)&h->part, sizeof(double) * nparts));
     CKS(alloc((void**)&h->ctrl, sizeof(Ctrl)));
-    CK(cudaMallocHost((void**)&h->hctrl, sizeof(Ctrl)));
-    memset(h->hctrl, 0, sizeof(Ctrl));
+    CK(cudaMallocHost((void**)&h->hctrl, sizeof(Ctrl) + 64));   // and the error word of tvcs_apply
+    memset(h->hctrl, 0, sizeof(Ctrl) + 64);
+    h->herr = reinterpret_cast<int*>(h->hctrl + 1);
     h->hctrl->algo = h->opt.algo;
     CK(cudaMemcpyAsync(h->ctrl, h->hctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemsetAsync(h->zeroN, 0, sizeof(float) * N, h->stream));
@@ -657,6 +649,25 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
         CKS(power_tau(h, h->opt.power_iters > 0 ? h->opt.power_iters : 100, &h->tau));
     }
     return sync_and_check(h, "tvcs_create");
+}
+
+// Whether p is memory of the handle's device (not host, managed or another GPU's memory).
+bool on_device(const tvcs_ctx* h, const void* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == h->dev;
+}
+
+bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
+bool apart(const void* a, size_t abytes, const void* b, size_t bbytes)
+{
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x + abytes <= y || y + bbytes <= x;
 }
 
 tvcs_status copy_in(tvcs_ctx* h, float* dst, const float* src, size_t count)
@@ -1120,14 +1131,42 @@ tvcs_status tvcs_apply(tvcs_handle h, const float* x, const float* y, float* r, 
 {
     CKS(check_handle(h));
     if (!x || !r || !g) return fail(TVCS_ERR_INVALID_ARG, "x, r and g must be non-NULL");
-    CKS(copy_in(h, h->tx, x, (size_t)h->N));
-    if (y) CKS(copy_in(h, h->ty, y, (size_t)h->m));
+    // Arrays in this device's memory go to the kernels as they are, where the kernels' 16-byte
+    // accesses allow it and no result overlaps another array; others through the handle's
+    // buffers.  (The regenerating products keep a table of the buffers they know.)
+    const size_t bm = sizeof(float) * (size_t)h->m, bN = sizeof(float) * (size_t)h->N;
+    const bool direct = !h->regen && on_device(h, x) && (!y || on_device(h, y)) && on_device(h, r) &&
+                        on_device(h, g) && aligned16(x) && aligned16(g) && apart(r, bm, g, bN) &&
+                        apart(r, bm, x, bN) && apart(g, bN, x, bN) &&
+                        (!y || (apart(r, bm, y, bm) && apart(g, bN, y, bm)));
+    const float* px = direct ? x : h->tx;
+    const float* py = !y ? nullptr : direct ? y : h->ty;
+    float* pr = direct ? r : h->tr;
+    float* pg = direct ? g : h->tg;
+    if (!direct) {
+        CKS(copy_in(h, h->tx, x, (size_t)h->N));
+        if (y) CKS(copy_in(h, h->ty, y, (size_t)h->m));
+    }
+    if (!h->use_q && !h->regen) {
+        // a bounded wait that gave up is recorded in a pinned word (the DCT products wait for nothing)
+        *h->herr = ERR_NONE;
+        products(h, px, py, pr, h->gpart2, pg, MODE_PLAIN, 0ull, 0, h->stream, 0, h->herr);
+        if (!direct) {
+            CKS(copy_out(h, r, h->tr, (size_t)h->m));
+            CKS(copy_out(h, g, h->tg, (size_t)h->N));
+        }
+        CKS(sync_and_check(h, "tvcs_apply"));
+        if (*static_cast<volatile int*>(h->herr) == ERR_TIMEOUT)
+            return fail(TVCS_ERR_TIMEOUT, "a bounded device wait gave up");
+        return TVCS_OK;
+    }
     // the kernels record a bounded wait that gave up in the control block's error word
     CK(cudaMemsetAsync(&h->ctrl->error, 0, sizeof(int), h->stream));
-    products(h, h->tx, y ? h->ty : nullptr, h->tr, h->gpart2, h->tg, MODE_PLAIN, 0ull, 0,
-             h->stream);
-    CKS(copy_out(h, r, h->tr, (size_t)h->m));
-    CKS(copy_out(h, g, h->tg, (size_t)h->N));
+    products(h, px, py, pr, h->gpart2, pg, MODE_PLAIN, 0ull, 0, h->stream);
+    if (!direct) {
+        CKS(copy_out(h, r, h->tr, (size_t)h->m));
+        CKS(copy_out(h, g, h->tg, (size_t)h->N));
+    }
     CKS(read_ctrl(h));
     if (h->hctrl->error == ERR_TIMEOUT)
         return fail(TVCS_ERR_TIMEOUT, "a bounded device wait gave up");

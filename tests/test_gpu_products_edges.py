@@ -52,3 +52,54 @@ def test_products_at_the_edges_of_the_row_split(tv, prec, n, m, with_y):
     gr = Ae.T @ r.astype(np.float64)
     scale_g = np.abs(Ae).T @ np.abs(r.astype(np.float64))
     assert np.all(np.abs(g - gr) <= 1e-5 * scale_g + 1e-30)
+
+
+@pytest.mark.parametrize("kind,n,m", [("fp32", 16, 77), ("fp32", 96, 921), ("fp8", 64, 701), ("cluster", 192, 500),
+                                      ("dct", 48, 461)])
+def test_apply_takes_every_kind_of_array(tv, kind, n, m):
+    """Arrays that the kernels may use as they are and arrays that go through the handle's buffers
+    (host memory, a start that is not 16-byte aligned, a result over an input or next to it)
+    give the same bits."""
+    N = n * n
+    g = torch.Generator(device="cuda").manual_seed(n + m)
+    opt = tv.tvcs_default_options()
+    opt.tau = 0.1
+    if kind == "dct":
+        rows = np.random.default_rng(m).choice(N, size=m, replace=False).astype(np.int32)
+        h = tv.tvcs_create_partial_dct(rows, n, 1.0, 1.0, 0.0, opt)
+    else:
+        opt.precision = tv.TVCS_PREC_FP8_BF16 if kind == "fp8" else tv.TVCS_PREC_FP32
+        h = tv.tvcs_create(torch.randn(m, N, generator=g, device="cuda") / m ** 0.5, 0, m, n, 1.0, 1.0, 0.0, opt)
+    x, y = torch.randn(N, generator=g, device="cuda"), torch.randn(m, generator=g, device="cuda")
+    r, gg = torch.empty_like(y), torch.empty_like(x)
+    tv.tvcs_apply(h, x, y, r, gg)
+
+    def odd(t):   # the same values from an address that is 4 bytes off
+        b = torch.empty(t.numel() + 1, device="cuda")
+        b[1:] = t
+        return b[1:]
+
+    def check(a, b):
+        for p, q in ((a, r), (b, gg)):
+            assert np.array_equal(p if isinstance(p, np.ndarray) else p.cpu().numpy(), q.cpu().numpy())
+
+    for xs, ys, ro, go in (
+            (x.cpu().numpy(), y, torch.empty_like(y), torch.empty_like(x)),
+            (x, y.cpu().numpy(), np.empty(m, np.float32), np.empty(N, np.float32)),
+            (odd(x), odd(y), odd(r), odd(gg)), (x, odd(y), odd(r), torch.empty_like(x))):
+        tv.tvcs_apply(h, xs, ys, ro, go)
+        check(ro, go)
+    # results over the inputs
+    x2, y2 = x.clone(), y.clone()
+    tv.tvcs_apply(h, x2, y2, y2, x2)
+    check(y2, x2)
+    # r and g in one buffer, g at an aligned place right after r's last entry
+    pad = (4 - m % 4) % 4
+    b = torch.zeros(pad + m + N, device="cuda")
+    tv.tvcs_apply(h, x, y, b[pad:pad + m], b[pad + m:])
+    check(b[pad:pad + m], b[pad + m:])
+    # no measurements: r = A x
+    tv.tvcs_apply(h, x, None, ro_ := torch.empty_like(y), torch.empty_like(x))
+    tv.tvcs_apply(h, x.cpu().numpy(), None, rh := np.empty(m, np.float32), np.empty(N, np.float32))
+    assert np.array_equal(ro_.cpu().numpy(), rh)
+    tv.tvcs_destroy(h)
