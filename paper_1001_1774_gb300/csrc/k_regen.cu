@@ -28,9 +28,8 @@
 // Many problems (own m, N, seed, x, y) share one launch.  Problem p's rows are
 // cut into chunks of a fixed number of rows (about 2^21 entries, and at least
 // 16 chunks when the problem has the rows: fixed by the problem, not by the
-// launch shape); the chunks of the active problems are numbered in problem
-// order, and cluster q of Q takes the chunks that start in the q-th of Q equal
-// shares of the active problems' entries.
+// launch shape); the chunks of the active problems are numbered in the order of
+// the problem table (largest chunks first), and the clusters take them in turn, there and back.
 // Every chunk stores its slice of A^T r and its ||r||^2 (added row after row)
 // in a slot of its own; k_regen_reduce adds a problem's slots in chunk order.
 // So every sum has an order fixed by the problem alone: the results do not
@@ -62,79 +61,50 @@ __host__ __device__ __forceinline__ int tile_rows_for(int W, int tile_cap)
     return rt;
 }
 
-// pre[p] = number of active chunks before problem p, pre[P] = T; prew[p] = entries
-// of A of the active problems before p, prew[P] = E (all threads).
-__device__ int active_prefix(const RegenProb* __restrict__ probs, int P, int mode, int* pre,
-                             int* scan, long long* prew, long long* wscan)
+// pre[p] = number of active chunks before problem p, pre[P] = T (all threads).
+__device__ int active_prefix(const RegenProb* __restrict__ probs, int P, int mode, int* pre, int* scan)
 {
     const int tid = threadIdx.x;
     int cnt[4];
-    long long wk[4];
     int local = 0;
-    long long wlocal = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int p = tid * 4 + k;
         int c = 0;
-        long long w = 0;
         if (p < P) {
             c = probs[p].chunks;
             if (mode == MODE_ITER && probs[p].ctrl && probs[p].ctrl->skip) c = 0;
-            if (c > 0) w = (long long)probs[p].m * probs[p].N;
         }
         cnt[k] = c;
-        wk[k] = w;
         local += c;
-        wlocal += w;
     }
     scan[tid] = local;
-    wscan[tid] = wlocal;
     __syncthreads();
     for (int off = 1; off < RG_THREADS; off <<= 1) {
         const int v = tid >= off ? scan[tid - off] : 0;
-        const long long wv = tid >= off ? wscan[tid - off] : 0;
         __syncthreads();
         scan[tid] += v;
-        wscan[tid] += wv;
         __syncthreads();
     }
     int run = scan[tid] - local;
-    long long wrun = wscan[tid] - wlocal;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int p = tid * 4 + k;
-        if (p < P) {
-            pre[p] = run;
-            prew[p] = wrun;
-        }
+        if (p < P) pre[p] = run;
         run += cnt[k];
-        wrun += wk[k];
     }
-    if (tid == RG_THREADS - 1) {
-        pre[P] = scan[tid];
-        prew[P] = wscan[tid];
-    }
+    if (tid == RG_THREADS - 1) pre[P] = scan[tid];
     __syncthreads();
     return pre[P];
 }
 
-// The first active chunk whose first entry lies at or after work offset t (T when
-// t is at or past the end).  Cluster q takes the chunks starting in
-// [q E / Q, (q+1) E / Q): ranges of equal work, whatever the chunk sizes.
-__device__ int chunk_at_work(const RegenProb* __restrict__ probs, int P, const int* pre,
-                             const long long* prew, long long t)
+// The k-th chunk of cluster q of Q: there and back over the clusters, so that with the largest
+// chunks first (the order of the problem table) the clusters' sums stay within about a chunk of
+// each other.  (Equal contiguous shares of the entries gave some clusters a large chunk and a
+// share of small ones: six problems of 114 M entries 0.52 ms a launch, here 0.40.)
+__device__ __forceinline__ int chunk_of(int k, int q, int Q)
 {
-    if (t >= prew[P]) return pre[P];
-    int lo = 0, hi = P - 1;   // the problem p with prew[p] <= t < prew[p+1]
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prew[mid] <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    const int p = lo;
-    const long long cw = (long long)probs[p].rows_per_chunk * probs[p].N;
-    const long long k = (t - prew[p] + cw - 1) / cw;
-    return pre[p] + (int)k;
+    return (k & 1) ? (k + 1) * Q - 1 - q : k * Q + q;
 }
 
 struct TileMeta {
@@ -163,9 +133,7 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
     extern __shared__ __align__(16) unsigned char smem[];
     int* pre = reinterpret_cast<int*>(smem);                    // pcap + 4 (pcap >= P, multiple of 4)
     int* scan = pre + pcap + 4;                                 // RG_THREADS
-    long long* prew = reinterpret_cast<long long*>(scan + RG_THREADS);   // pcap + 4
-    long long* wscan = prew + pcap + 4;                         // RG_THREADS
-    float* gs = reinterpret_cast<float*>(wscan + RG_THREADS);   // A^T r slice, wmax
+    float* gs = reinterpret_cast<float*>(scan + RG_THREADS);    // A^T r slice, wmax
     float* tile = gs + wmax;                                    // NBUF x tile_cap
     float* wpart = tile + NBUF * tile_cap;                      // 2 x RTMAX x SEGMAX, this block's
     float* slotv = wpart + 2 * RG_RTMAX * RG_SEGMAX;            // the same, read by the peers
@@ -179,13 +147,11 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int segs = RG_NSEG / CS;   // segments of a row this block owns
 
-    active_prefix(probs, P, mode, pre, scan, prew, wscan);
+    const int T = active_prefix(probs, P, mode, pre, scan);
     if (blockIdx.x == 0)
         for (int p = tid; p <= P; p += RG_THREADS) pre_out[p] = pre[p];
-    const long long E = prew[P];
-    int j = chunk_at_work(probs, P, pre, prew, (long long)cq * E / Q);
-    const int j1 = chunk_at_work(probs, P, pre, prew, (long long)(cq + 1) * E / Q);
-    if (j >= j1) return;   // the whole cluster has no chunk
+    int jk = 0, j = chunk_of(0, cq, Q);
+    if (j >= T) return;   // the whole cluster has no chunk
 
     for (int i = tid; i < wmax; i += RG_THREADS) gs[i] = 0.f;
 
@@ -244,7 +210,7 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
     TileMeta prev{};
     bool have_prev = false;
     for (int t = 0;; ++t) {
-        const bool have_cur = j < j1;
+        const bool have_cur = j < T;
         const int sb = t & 1;                  // partial-dot and r buffers
         const int tb = NBUF == 2 ? sb : 0;     // tile buffer
         TileMeta cur{};
@@ -305,13 +271,11 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
             row += cur.nr;
             cur.last = row >= cend ? 1 : 0;
             if (row >= cend) {
-                ++j;
-                if (j < j1) {
-                    ++c;
-                    if (j >= pre[p + 1]) {   // first chunk of the next active problem
+                j = chunk_of(++jk, cq, Q);
+                if (j < T) {
+                    if (j >= pre[p + 1]) {   // a chunk of a later active problem
                         do ++p;
                         while (pre[p + 1] <= j);
-                        c = j - pre[p];
                         pr = probs + p;
                         N = pr->N;
                         m = pr->m;
@@ -319,6 +283,7 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
                         W = N / CS;
                         rt = tile_rows_for(W, tile_cap);
                     }
+                    c = j - pre[p];
                     row = c * RC;
                     cend = min(m, row + RC);
                 }
@@ -347,9 +312,13 @@ k_regen_products(const RegenProb* __restrict__ probs, int P, int mode, int wmax,
     cluster_wait();
 }
 
-// g = sum of the chunk slots in chunk order, ctrl->r2 = sum of the chunk r2 slots.
-// Grid (ceil(maxN / 1024), P), 256 threads, one float4 per thread.
-__global__ void __launch_bounds__(256)
+// g = sum of the chunk slots in chunk order, ctrl->r2 = sum of the chunk r2 slots in chunk order.
+// Grid (ceil(maxN / 256), P), 64 threads, one float4 per thread with eight slots' loads in
+// flight (one load after the other took 8 us at 40 chunks); the r2 slots are loaded by a warp and
+// added by its lane 0.
+constexpr int RR_THREADS = 64;
+
+__global__ void __launch_bounds__(RR_THREADS)
 k_regen_reduce(const RegenProb* __restrict__ probs, int P, const int* __restrict__ pre,
                cudaGraphConditionalHandle cond, int set_cond)
 {
@@ -365,30 +334,40 @@ k_regen_reduce(const RegenProb* __restrict__ probs, int P, const int* __restrict
     const int K = pre[p + 1] - pre[p];
     if (K == 0) return;   // inactive in this launch
     const int n4 = pr.N / 4;
-    const int q4 = blockIdx.x * blockDim.x + tid;
+    const int q4 = blockIdx.x * RR_THREADS + tid;
     if (q4 < n4) {
         const float4* slot = reinterpret_cast<const float4*>(pr.gslot);
         float4 acc = slot[q4];
-        for (int h = 1; h < K; ++h) {
-            const float4 v = slot[(size_t)h * n4 + q4];
-            acc.x += v.x;
-            acc.y += v.y;
-            acc.z += v.z;
-            acc.w += v.w;
+        for (int h0 = 1; h0 < K; h0 += 8) {
+            float4 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (h0 + k < K) v[k] = slot[(size_t)(h0 + k) * n4 + q4];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (h0 + k < K) {
+                    acc.x += v[k].x;
+                    acc.y += v[k].y;
+                    acc.z += v[k].z;
+                    acc.w += v[k].w;
+                }
         }
         reinterpret_cast<float4*>(pr.g)[q4] = acc;
     }
-    if (blockIdx.x == 0 && tid == 0 && pr.ctrl) {
-        float2 v = pr.r2slot[0];
-        for (int h = 1; h < K; ++h) v = ds_add(v, pr.r2slot[h]);
-        pr.ctrl->r2 = ds_value(v);
+    if (blockIdx.x == 0 && tid < 32 && pr.ctrl) {
+        float2 t = pr.r2slot[0];
+        for (int h0 = 1; h0 < K; h0 += 32) {
+            const float2 v = h0 + tid < K ? pr.r2slot[h0 + tid] : make_float2(0.f, 0.f);
+            for (int k = 0; k < 32 && h0 + k < K; ++k)
+                t = ds_add(t, make_float2(__shfl_sync(0xffffffffu, v.x, k), __shfl_sync(0xffffffffu, v.y, k)));
+        }
+        if (tid == 0) pr.ctrl->r2 = ds_value(t);
     }
 }
 
 static size_t regen_smem(int wmax, int tile_cap, int nbuf, int pcap)
 {
     return sizeof(int) * ((size_t)pcap + 4 + RG_THREADS) +
-           sizeof(long long) * ((size_t)pcap + 4 + RG_THREADS) +
            sizeof(float) * ((size_t)wmax + (size_t)nbuf * tile_cap + 4 * RG_RTMAX * RG_SEGMAX +
                             2 * RG_RTMAX);
 }
@@ -482,8 +461,8 @@ void launch_regen_reduce(const RegenProb* probs, int P, int maxN, int mode, cons
 {
     (void)mode;
     (void)plan;
-    const dim3 grid((maxN / 4 + 255) / 256, P);
-    k_regen_reduce<<<grid, 256, 0, s>>>(probs, P, pre, (cudaGraphConditionalHandle)cond, set_cond);
+    const dim3 grid((maxN / 4 + RR_THREADS - 1) / RR_THREADS, P);
+    k_regen_reduce<<<grid, RR_THREADS, 0, s>>>(probs, P, pre, (cudaGraphConditionalHandle)cond, set_cond);
 }
 
 }  // namespace tvcs
