@@ -89,9 +89,12 @@ struct tvcs_ctx {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphExec_t tail[16] = {};
-    // the loop as one launch (n <= 96, stored A): blocks (0: the graphs above), exchange
-    // buffers, tags used so far
+    // the loop as one launch (n <= 96, stored A): blocks (0: the graphs above), whether A stays on
+    // chip (launch_loop_reg); blocks of the power iteration's launch (0: a launch per product);
+    // exchange buffers, tags used so far
     int loop_grid = 0;
+    bool loop_reg = false;
+    int power_grid = 0;
     uint64_t *ubuf = nullptr, *colx = nullptr, *rowx = nullptr, *nbuf = nullptr;
     uint32_t loop_tag = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;

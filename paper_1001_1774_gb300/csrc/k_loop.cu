@@ -2,9 +2,10 @@
 // iteration and the test of eq. (stop)) as ONE persistent cooperative launch, for images
 // up to 96 x 96 with a stored A (Xiao & Yang, Sec. 2.1-2.2).
 //
-// G blocks, one per SM.  Block b owns a contiguous range of rows of A for the two products
-// (as in k_products.cu: a ring of pieces filled by bulk copies, a row's columns in
-// registers for both uses).  The first n/2 blocks also carry the u-step: block j owns the
+// G blocks, one per SM.  Block b owns a contiguous range of rows of A for the two products.  At
+// n <= 64 these stay on chip for the whole launch where they fit, as binary32: 8 to 32 of them in
+// registers, the rest in shared memory (k_loop_reg).  Otherwise (k_loop) they come through a
+// ring of pieces filled by bulk copies, as in k_products.cu.  The first n/2 blocks also carry the u-step: block j owns the
 // image rows 2j and 2j+1 and column slot j of the half spectrum (slot 0: the two real
 // columns 0 and n/2 packed as one complex column).  An iteration:
 //   1  blocks j: lambda update, shrink and D^T y of their rows (one halo row recomputed),
@@ -22,14 +23,17 @@
 // iterations; a buffer is written again only after its readers have passed a later exchange.
 //
 // What bounds it: the exchanges between blocks (1 to 1.5 us each through L2: partials, column
-// slots, rows, u), as the ring holds every row of A at n <= 64 and A is read once per launch.
-// The chain of two launches per iteration that it replaces (u-solve cluster, products) paid
-// two kernel boundaries, a grid barrier with a global reduction and a second read of g.  Per
-// iteration, 200 iterations: n = 16 (m = 77) 9.6 -> 6.8 us, n = 32 (307) 11.7 -> 7.9, n = 48
-// (691) 12.5 -> 9.0, n = 64 (1229) 14.75 -> 11.4 (bf16 hi + lo 17 -> 13.5), n = 96 (921) 17.0
-// -> 16.3, n = 96 (2765) 23.7 -> 23.3; and no loop graphs to build.  At n = 128 it measured
-// 52.5 us against 52.1 (u-solve and exchanges take 13 us in which L2 cannot hold more of A
-// than the row order already keeps there), so that size keeps the chain.
+// slots, rows, u), and at n = 96 reading A.  The chain of two launches per iteration that it
+// replaces (u-solve cluster, products) paid two kernel boundaries, a grid barrier with a
+// global reduction and a second read of g, and had loop graphs to build.  us an iteration, 200
+// iterations, binary32, as the chain -> k_loop -> k_loop_reg:
+//   n = 16 (m = 77) 9.6 -> 6.7 -> 4.8, n = 32 (307) 11.7 -> 7.8 -> 7.3, n = 48 (691) 12.5 -> 8.7 ->
+//   8.0, n = 64 (1229) 14.75 -> 11.4 -> 9.7 (2048: 13.2 -> 10.0; fp8, 1229: 13.8 -> 9.7), n = 96
+//   (921) 17.0 -> 16.3, n = 96 (2765) 23.7 -> 23.3.
+// (From the ring a pass over 9 rows took three steps of 1.3 us, each a wait, a decode, a warp
+// reduction and a block barrier in series; from registers all rows share one of each.)  At
+// n = 128 k_loop measured 52.5 us against 52.1 (u-solve and exchanges take 13 us in which L2 cannot
+// hold more of A than the row order already keeps there), so that size keeps the chain.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,40 +41,14 @@
 #include "common.cuh"
 #include "fft.cuh"
 #include "kernels.h"
+#include "loop_exchange.cuh"
+#include "loop_rows.cuh"
 #include "products.cuh"
 #include "usolve_steps.cuh"
 
 namespace tvcs {
 
 namespace {
-
-// Tagged words: value in the low half, tag in the high half.
-__device__ __forceinline__ uint64_t tagged(float v, uint32_t tag)
-{
-    return ((uint64_t)tag << 32) | __float_as_uint(v);
-}
-
-__device__ __forceinline__ void send2(uint64_t* p, float a, float b, uint32_t tag)
-{
-    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(tagged(a, tag)),
-                 "l"(tagged(b, tag))
-                 : "memory");
-}
-
-__device__ __forceinline__ ulonglong2 peek2(const uint64_t* p)
-{
-    ulonglong2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p)
-                 : "memory");
-    return v;
-}
-
-__device__ __forceinline__ bool has_tag(ulonglong2 v, uint32_t tag)
-{
-    return (uint32_t)(v.x >> 32) == tag && (uint32_t)(v.y >> 32) == tag;
-}
-
-__device__ __forceinline__ float word_f(uint64_t v) { return __uint_as_float((uint32_t)v); }
 
 // A block's scalars, in shared memory: what a section needs it reads again, so that no value
 // stays in a register through the products' loop (at n = 128 its rows, u and sums take 96 of
@@ -81,6 +59,7 @@ struct LoopState {
     int pending;             // the multiplier update of the last u is due
     int algo;
     int i0, nrows;           // this block's rows of A
+    int last;                // this block is the last to end
     double du2, u2, tol;     // norms of the last iteration, eq. (stop)
 };
 
@@ -96,41 +75,12 @@ struct Ring {
     int pass, o, slot, phase;         // next piece to issue, its slot and the slot's phase
 };
 
-__device__ __forceinline__ int fresh_tid()   // not kept from one section to the next
-{
-    int t;
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
-    return t;
-}
-
-// Bound of a block's waits, and its record that one gave up.
-struct Waits {
-    long long budget;
-    volatile int* gave_up;   // shared memory
-};
-
-// The two words at p once both carry `tag` (v: a first look at them); whatever is there
-// when the budget runs out or another wait of the block has given up.
-__device__ __forceinline__ ulonglong2 await2(const uint64_t* p, uint32_t tag, ulonglong2 v, const Waits& w)
-{
-    if (has_tag(v, tag)) return v;
-    const long long t0 = clock64();
-    for (;;) {
-        v = peek2(p);
-        if (has_tag(v, tag)) return v;
-        if (*w.gave_up) return v;
-        if (clock64() - t0 > w.budget) {
-            *w.gave_up = 1;
-            return v;
-        }
-    }
-}
-
 template <int NN_, int PREC_, int TC_, int VW_, int V_, int RL_, int RB_, int RP_, int NPC_>
 struct LoopShape {
     using P = ProdShape<PREC_, TC_, VW_, V_, RL_, RB_, 2>;
     static_assert(P::N == NN_ * NN_, "columns");
-    static constexpr int NN = NN_, PREC = PREC_, TC = TC_, VW = VW_, V = V_, RL = RL_, RB = RB_;
+    static constexpr int NN = NN_, PREC = PREC_, TC = TC_, VW = VW_, V = V_, RL = RL_, RB = RB_, RREG = 0;
+    static constexpr int CP = P::CPT / 2;
     static constexpr int N = P::N, THREADS = P::THREADS, WARPS = P::WARPS, RS = P::RS, WPR = P::WPR;
     static constexpr int B0 = P::B0, B1 = P::B1;
     static constexpr int RP = RP_, Q = RS / RP, NPC = NPC_;   // rows a piece, pieces a step, pieces in the ring
@@ -155,13 +105,50 @@ struct LoopShape {
     static constexpr size_t O_Y2 = O_Y1 + 2 * NN * 4;                      // rows 2j-1 .. 2j+1
     static constexpr size_t O_G = O_Y2 + 3 * NN * 4;                       // g of rows 2j, 2j+1
     static constexpr size_t O_GS = O_G + 2 * NN * 4;                       // [GG][GC] float4
-    static constexpr size_t O_FA = O_GS + (size_t)GG * GC * 16;            // two transforms
+    static constexpr size_t GS = (size_t)GG * GC * 16;
+    static constexpr size_t O_FA = O_GS + GS;                              // two transforms
     static constexpr size_t O_FB = O_FA + NN * 8;
     static constexpr size_t O_TW = O_FB + NN * 8;
     static constexpr size_t O_RD = O_TW + NN * 8;                          // rdiv of the slot and of column n/2
     static constexpr size_t SMEM = O_RD + 2 * NN * 4;
     static_assert(GG >= 1 && THREADS % 32 == 0 && THREADS >= 96 && NN % 4 == 0, "threads");
     static_assert(SMEM <= 227 * 1024, "shared memory");
+};
+
+// The same without a ring: every row of A on chip as binary32 for the whole launch, RL RREG of
+// them in registers (a thread has its columns of RREG rows), up to XMAX more in shared memory.
+template <int NN_, int TC_, int V_, int RL_, int RREG_>
+struct RegShape {
+    static constexpr int NN = NN_, PREC = 0, TC = TC_, VW = 4, V = V_, RL = RL_, RREG = RREG_;
+    static constexpr int N = NN * NN, THREADS = TC * RL, WARPS = THREADS / 32, WPR = TC / 32, CP = VW * V / 2;
+    static_assert(TC * VW * V == N && TC % 32 == 0 && RREG % 4 == 0 && THREADS >= 96 && THREADS <= 512, "split");
+    static constexpr int NP = NN / 2, GC = 2 * NN / 4, GG = THREADS / GC, WL = 3 * NN;
+    static constexpr int RROWS = RL * RREG;
+    static constexpr int RED = WPR | 1;           // stride of a row's warp sums (odd banks)
+    static constexpr size_t al(size_t b) { return (b + 15) / 16 * 16; }
+    static constexpr size_t O_DRED = 0;           // [32] float2
+    static constexpr size_t O_STATE = O_DRED + 32 * 8;
+    static constexpr size_t O_SU = O_STATE + al(sizeof(LoopState));       // as in LoopShape
+    static constexpr size_t O_WL = O_SU + 4 * NN * 4;
+    static constexpr size_t O_Y1 = O_WL + 2 * 4 * WL * 4;
+    static constexpr size_t O_Y2 = O_Y1 + 2 * NN * 4;
+    static constexpr size_t O_G = O_Y2 + 3 * NN * 4;
+    static constexpr size_t O_GS = O_G + 2 * NN * 4;
+    static constexpr size_t GS = std::max((size_t)GG * GC * 16, (size_t)(RL - 1) * N * 4);
+    static constexpr size_t O_FA = O_GS + GS;
+    static constexpr size_t O_FB = O_FA + NN * 8;
+    static constexpr size_t O_TW = O_FB + NN * 8;
+    static constexpr size_t O_RD = O_TW + NN * 8;
+    static constexpr size_t O_RED = O_RD + 2 * NN * 4;
+    static constexpr size_t ROW_BYTES = (size_t)RED * 4 + 8;   // a row's warp sums, r and f
+    static constexpr size_t LIMIT = 227 * 1024;
+    static constexpr int XMAX = (int)((LIMIT - O_RED - 64 - RROWS * ROW_BYTES) / ((size_t)N * 4 + ROW_BYTES));
+    static constexpr int RMAX = RROWS + XMAX, YMAX = RMAX;
+    static constexpr size_t O_R = al(O_RED + (size_t)RMAX * RED * 4);
+    static constexpr size_t O_Y = al(O_R + (size_t)RMAX * 4);
+    static constexpr size_t O_A = al(O_Y + (size_t)RMAX * 4);
+    static constexpr size_t smem(int rows) { return O_A + (size_t)std::max(0, rows - RROWS) * N * 4; }
+    static_assert(GG >= 1 && smem(RMAX) <= LIMIT, "shared memory");
 };
 
 #define LOOP_SMEM extern __shared__ __align__(128) unsigned char smem[]
@@ -387,13 +374,122 @@ __device__ __forceinline__ void loop_ustep(const LoopArgs& q, int it)
     }
 }
 
+// u of iteration `it` into the thread's registers, and in the u-step's blocks the rows
+// 2j-1 .. 2j+2 for the next w-step.
+template <class S>
+__device__ __forceinline__ void loop_take_u(const LoopArgs& q, int it, uint64_t* xu)
+{
+    LOOP_SMEM;
+    constexpr int NN = S::NN, TC = S::TC, VW = S::VW, V = S::V, N = S::N;
+    LoopState* st = LOOP_AT(LoopState, S::O_STATE);
+    const Waits waits{q.budget, &st->gave_up};
+    const int tid = fresh_tid();
+    const int ltid = tid % TC;
+    const uint32_t tag = q.tag0 + (uint32_t)it;
+    const uint64_t* ubuf = q.ubuf + (size_t)(it & 1) * N;
+    {
+        constexpr int W2 = VW / 2;   // two-word packets per vector
+        const uint64_t* xb = ubuf + (size_t)ltid * VW;
+        // one packet first: while u is awaited only that one is polled
+        const ulonglong2 v0 = await2(xb, tag, peek2(xb), waits);
+        xu[0] = pack2(word_f(v0.x), word_f(v0.y));
+        constexpr int NV = V * W2;
+        constexpr int BATCH = 8;
+    #pragma unroll
+        for (int b = 1; b < NV; b += BATCH) {
+            ulonglong2 v[BATCH];
+            auto look = [&]() {   // the batch's packets; true once every one has arrived
+                bool all = true;
+    #pragma unroll
+                for (int k = 0; k < BATCH; ++k)
+                    if (b + k < NV) v[k] = peek2(xb + (size_t)((b + k) / W2) * TC * VW + 2 * ((b + k) % W2));
+    #pragma unroll
+                for (int k = 0; k < BATCH; ++k)
+                    if (b + k < NV) all = all && has_tag(v[k], tag);
+                return all;
+            };
+            if (!look()) {
+                const long long t0 = clock64();
+                while (!look()) {
+                    if (*waits.gave_up) break;
+                    if (clock64() - t0 > waits.budget) {
+                        *waits.gave_up = 1;
+                        break;
+                    }
+                }
+            }
+    #pragma unroll
+            for (int k = 0; k < BATCH; ++k)
+                if (b + k < NV) xu[b + k] = pack2(word_f(v[k].x), word_f(v[k].y));
+        }
+    }
+    if (blockIdx.x < S::NP) {   // rows 2j-1 .. 2j+2 for the next w-step (warp 0 has read the old ones)
+        float* su = LOOP_AT(float, S::O_SU);
+        const int r0 = 2 * blockIdx.x;
+        __syncthreads();
+        for (int i = 2 * tid; i < 4 * NN; i += 2 * S::THREADS) {
+            const int rr = i / NN, c = i - rr * NN;
+            const uint64_t* p = ubuf + ((r0 - 1 + rr + NN) % NN) * NN + c;
+            const ulonglong2 v = await2(p, tag, peek2(p), waits);
+            su[i] = word_f(v.x);
+            su[i + 1] = word_f(v.y);
+        }
+    }
+}
+
+// The block's partial of A^T r to global memory.
+template <class S>
+__device__ __forceinline__ void loop_partial(const LoopArgs& q, uint64_t* acc)
+{
+    LOOP_SMEM;
+    constexpr int TC = S::TC, VW = S::VW, V = S::V, RL = S::RL, N = S::N, VP = VW / 2;
+    [[maybe_unused]] constexpr int CP = S::CP;
+    const int tid = fresh_tid();
+    const int lane_row = tid / TC;
+    const int ltid = tid - lane_row * TC;
+    if constexpr (RL > 1) {   // the row lanes' sums meet in the scratch of g
+        float* scr = LOOP_AT(float, S::O_GS);
+        static_assert((size_t)(RL - 1) * N * 4 <= S::GS, "the lanes' sums fit");
+        if (lane_row > 0) {
+#pragma unroll
+            for (int c = 0; c < CP; ++c)
+                *reinterpret_cast<uint64_t*>(scr + (size_t)(lane_row - 1) * N + (ltid + (c / VP) * TC) * VW +
+                                             2 * (c % VP)) = acc[c];
+        }
+        __syncthreads();
+        if (lane_row == 0) {
+#pragma unroll
+            for (int c = 0; c < CP; ++c)
+                for (int l = 1; l < RL; ++l)
+                    acc[c] = add2(acc[c],
+                                  *reinterpret_cast<const uint64_t*>(scr + (size_t)(l - 1) * N +
+                                                                     (ltid + (c / VP) * TC) * VW + 2 * (c % VP)));
+        }
+    }
+    if (lane_row == 0) {
+        float* out = q.gpart + (size_t)blockIdx.x * N;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            float* ov = out + (ltid + v * TC) * VW;
+            if constexpr (VW % 4 == 0) {
+#pragma unroll
+                for (int k = 0; k < VW / 4; ++k)
+                    reinterpret_cast<ulonglong2*>(ov)[k] =
+                        make_ulonglong2(acc[v * VP + 2 * k], acc[v * VP + 2 * k + 1]);
+            } else {
+                *reinterpret_cast<uint64_t*>(ov) = acc[v];
+            }
+        }
+    }
+}
+
 // One pass: u into registers, r = A u - f and the partial of A^T r over this block's rows,
 // to global memory.
 template <class S>
 __device__ __forceinline__ void loop_pass(const LoopArgs& q, int it)
 {
     LOOP_SMEM;
-    constexpr int NN = S::NN, PREC = S::PREC, TC = S::TC, VW = S::VW, V = S::V, RL = S::RL, RB = S::RB;
+    constexpr int PREC = S::PREC, TC = S::TC, VW = S::VW, V = S::V, RB = S::RB;
     constexpr int N = S::N, RS = S::RS, WPR = S::WPR, CP = S::P::CPT / 2, VP = VW / 2, Q = S::Q;
     uint64_t* full = LOOP_AT(uint64_t, S::O_BAR);
     float* red = LOOP_AT(float, S::O_RED);
@@ -402,59 +498,9 @@ __device__ __forceinline__ void loop_pass(const LoopArgs& q, int it)
     const int tid = fresh_tid();
     const int lane_row = tid / TC;
     const int ltid = tid - lane_row * TC;
-    const uint32_t tag = q.tag0 + (uint32_t)it;
-    const uint64_t* ubuf = q.ubuf + (size_t)(it & 1) * N;
 
-    // ---------------- u ----------------
     uint64_t xu[CP], acc[CP];
-        {
-            constexpr int W2 = VW / 2;   // two-word packets per vector
-            const uint64_t* xb = ubuf + (size_t)ltid * VW;
-            // one packet first: while u is awaited only that one is polled
-            const ulonglong2 v0 = await2(xb, tag, peek2(xb), waits);
-            xu[0] = pack2(word_f(v0.x), word_f(v0.y));
-            constexpr int NV = V * W2;
-            constexpr int BATCH = 8;
-    #pragma unroll
-            for (int b = 1; b < NV; b += BATCH) {
-                ulonglong2 v[BATCH];
-                auto look = [&]() {   // the batch's packets; true once every one has arrived
-                    bool all = true;
-    #pragma unroll
-                    for (int k = 0; k < BATCH; ++k)
-                        if (b + k < NV) v[k] = peek2(xb + (size_t)((b + k) / W2) * TC * VW + 2 * ((b + k) % W2));
-    #pragma unroll
-                    for (int k = 0; k < BATCH; ++k)
-                        if (b + k < NV) all = all && has_tag(v[k], tag);
-                    return all;
-                };
-                if (!look()) {
-                    const long long t0 = clock64();
-                    while (!look()) {
-                        if (*waits.gave_up) break;
-                        if (clock64() - t0 > waits.budget) {
-                            *waits.gave_up = 1;
-                            break;
-                        }
-                    }
-                }
-    #pragma unroll
-                for (int k = 0; k < BATCH; ++k)
-                    if (b + k < NV) xu[b + k] = pack2(word_f(v[k].x), word_f(v[k].y));
-            }
-        }
-        if (blockIdx.x < S::NP) {   // rows 2j-1 .. 2j+2 for the next w-step (warp 0 has read the old ones)
-            float* su = LOOP_AT(float, S::O_SU);
-            const int r0 = 2 * blockIdx.x;
-            __syncthreads();
-            for (int i = 2 * tid; i < 4 * NN; i += 2 * S::THREADS) {
-                const int rr = i / NN, c = i - rr * NN;
-                const uint64_t* p = ubuf + ((r0 - 1 + rr + NN) % NN) * NN + c;
-                const ulonglong2 v = await2(p, tag, peek2(p), waits);
-                su[i] = word_f(v.x);
-                su[i + 1] = word_f(v.y);
-            }
-        }
+    loop_take_u<S>(q, it, xu);
 #pragma unroll
     for (int c = 0; c < CP; ++c) acc[c] = 0ull;
     float2 r2 = make_float2(0.f, 0.f);   // double-single ||r||^2 of this lane's rows (ltid == 0)
@@ -571,42 +617,24 @@ __device__ __forceinline__ void loop_pass(const LoopArgs& q, int it)
         }
     }
 
-    // ---------------- partial of A^T r ----------------
     if (ltid == 0) LOOP_AT(float2, S::O_DRED)[lane_row] = r2;
-    if constexpr (RL > 1) {   // the row lanes' sums meet in the scratch of g
-        float* scr = LOOP_AT(float, S::O_GS);
-        static_assert((size_t)(RL - 1) * N * 4 <= (size_t)S::GG * S::GC * 16, "the lanes' sums fit");
-        if (lane_row > 0) {
-#pragma unroll
-            for (int c = 0; c < CP; ++c)
-                *reinterpret_cast<uint64_t*>(scr + (size_t)(lane_row - 1) * N + (ltid + (c / VP) * TC) * VW +
-                                             2 * (c % VP)) = acc[c];
-        }
-        __syncthreads();
-        if (lane_row == 0) {
-#pragma unroll
-            for (int c = 0; c < CP; ++c)
-                for (int l = 1; l < RL; ++l)
-                    acc[c] = add2(acc[c],
-                                  *reinterpret_cast<const uint64_t*>(scr + (size_t)(l - 1) * N +
-                                                                     (ltid + (c / VP) * TC) * VW + 2 * (c % VP)));
-        }
-    }
-    if (lane_row == 0) {
-        float* out = q.gpart + (size_t)blockIdx.x * N;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            float* ov = out + (ltid + v * TC) * VW;
-            if constexpr (VW % 4 == 0) {
-#pragma unroll
-                for (int k = 0; k < VW / 4; ++k)
-                    reinterpret_cast<ulonglong2*>(ov)[k] =
-                        make_ulonglong2(acc[v * VP + 2 * k], acc[v * VP + 2 * k + 1]);
-            } else {
-                *reinterpret_cast<uint64_t*>(ov) = acc[v];
-            }
-        }
-    }
+    loop_partial<S>(q, acc);
+}
+
+// The same pass over rows that stay on chip (RegShape).
+template <class S>
+__device__ __forceinline__ void loop_pass_reg(const LoopArgs& q, int it, const uint64_t (&a)[S::RREG][S::CP])
+{
+    LOOP_SMEM;
+    const int nrows = *(volatile const int*)&LOOP_AT(LoopState, S::O_STATE)->nrows;
+    const float* srow = LOOP_AT(float, S::O_A);
+    float* sr = LOOP_AT(float, S::O_R);
+    const int tid = fresh_tid(), lane_row = tid / S::TC, ltid = tid - lane_row * S::TC;
+    uint64_t xu[S::CP], acc[S::CP];
+    loop_take_u<S>(q, it, xu);
+    reg_residual<S>(a, xu, srow, LOOP_AT(float, S::O_Y), LOOP_AT(float, S::O_RED), sr, nrows, tid);
+    reg_adjoint<S>(a, srow, sr, nrows, lane_row, ltid, acc);
+    loop_partial<S>(q, acc);
 }
 
 // After a pass: thread 0 arrives and, in the u-step's blocks, waits for all partials; warp 1
@@ -623,10 +651,12 @@ __device__ __forceinline__ void loop_arrive(const LoopArgs& q, int it)
     const Waits waits{q.budget, &st->gave_up};
     if (warp == 0) {
         if (lane == 0) {
-            const float2* dred = LOOP_AT(float2, S::O_DRED);
-            float2 s = dred[0];
-            for (int l = 1; l < S::RL; ++l) s = ds_add(s, dred[l]);
-            q.r2part[blk] = s;
+            if constexpr (S::RREG == 0) {
+                const float2* dred = LOOP_AT(float2, S::O_DRED);
+                float2 s = dred[0];
+                for (int l = 1; l < S::RL; ++l) s = ds_add(s, dred[l]);
+                q.r2part[blk] = s;
+            }
             __threadfence();
             atomicAdd(&q.ctrl->lbar, 1ull);
             if (ublk) {
@@ -674,7 +704,7 @@ __device__ __forceinline__ void loop_gather(const LoopArgs& q)
     const int col = tid % GC, grp = tid / GC;
     if (grp < GG) {
         const float4* gp = reinterpret_cast<const float4*>(q.gpart) + (size_t)2 * blockIdx.x * S::NN / 4 + col;
-        constexpr int BATCH = 10;
+        constexpr int BATCH = S::RREG > 0 ? 152 / GG + 1 : 10;   // (loads in flight; one batch on 152 SMs)
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int p0 = grp; p0 < G; p0 += GG * BATCH) {
             float4 v[BATCH];
@@ -713,15 +743,17 @@ __device__ __forceinline__ void loop_begin(const LoopArgs& q)
     const int nrows = (int)(((long long)q.m * (blk + 1)) / gridDim.x) - i0;
     LoopState* st = LOOP_AT(LoopState, S::O_STATE);
     if (tid == 0) {
-        uint64_t* full = LOOP_AT(uint64_t, S::O_BAR);
-        for (int s = 0; s < S::NPC; ++s) mbar_init(&full[s], 1);
-        fence_mbar_init();
         st->gave_up = st->end = 0;
         st->pending = q.ctrl->pending;
         st->algo = q.ctrl->algo;
         st->i0 = i0;
         st->nrows = nrows;
         st->tol = q.ctrl->tol;
+    }
+    if constexpr (S::RREG == 0) if (tid == 0) {
+        uint64_t* full = LOOP_AT(uint64_t, S::O_BAR);
+        for (int s = 0; s < S::NPC; ++s) mbar_init(&full[s], 1);
+        fence_mbar_init();
         Ring& g = *LOOP_AT(Ring, S::O_RING);
         g.p0 = q.P0 + (size_t)i0 * N * S::B0;
         g.p1 = S::B1 > 0 ? q.P1 + (size_t)i0 * N * S::B1 : nullptr;
@@ -792,9 +824,23 @@ __device__ __forceinline__ void loop_end(const LoopArgs& q, int it)
             q.lam[wi] = src[2 * WL + NN + i];
             q.lam[wi + N] = src[3 * WL + NN + i];
         }
-        if (blk == 0) {
+    }
+    bool ends = blk == 0;   // this block writes the control block
+    if constexpr (S::RREG > 0) {   // r of the block's rows and its norm; the last block to come adds the norms
+        const float* sr = LOOP_AT(float, S::O_R);
+        float2 v = make_float2(0.f, 0.f);
+        for (int i = tid; i < st->nrows; i += S::THREADS) {
+            q.r[st->i0 + i] = sr[i];
+            v = ds_add(v, ds_sq(sr[i]));
+        }
+        v = block_sum_ds(v, LOOP_AT(float2, S::O_DRED));
+        if (tid == 0) q.r2part[blk] = v;
+        ends = last_block_all(&ctrl->ticket_gather, &st->last);
+    }
+    if (!__syncthreads_or(st->gave_up)) {
+        if (ends) {
             // ||r||^2 = sum of the G partials, fixed order (every partial is visible: the
-            // arrivals of this iteration were awaited)
+            // arrivals of this iteration were awaited, or this block is the last)
             float2* dred = LOOP_AT(float2, S::O_DRED);
             float2 v = make_float2(0.f, 0.f);
             for (int p = tid; p < (int)gridDim.x; p += S::THREADS) v = ds_add(v, __ldcg(q.r2part + p));
@@ -815,7 +861,7 @@ __device__ __forceinline__ void loop_end(const LoopArgs& q, int it)
             }
         }
     }
-    if (tid == 0) {   // let the copies still in flight land (bounded): every slot's last phase
+    if constexpr (S::RREG == 0) if (tid == 0) {   // let the copies still in flight land (bounded): every slot's last phase
         const Ring& g = *LOOP_AT(Ring, S::O_RING);
         const int used = g.passes == 1 ? min(S::NPC, g.pieces) : g.passes > 1 ? S::NPC : 0;
         uint64_t* full = LOOP_AT(uint64_t, S::O_BAR);
@@ -841,6 +887,32 @@ __global__ void __maxnreg__(128) k_loop(const __grid_constant__ LoopArgs q)
         __syncthreads();
         loop_arrive<S>(q, it);
         // (the vote makes the outcome the same for every thread of the block)
+        if (__syncthreads_or(st->gave_up)) break;
+        const int end = st->end;
+        if (blockIdx.x < S::NP) loop_gather<S>(q);
+        if (end) break;
+    }
+    loop_end<S>(q, it);
+}
+
+template <int NN, int TC, int V, int RL, int RREG>
+__global__ void __launch_bounds__(TC * RL, 1) k_loop_reg(const __grid_constant__ LoopArgs q)
+{
+    using S = RegShape<NN, TC, V, RL, RREG>;
+    LOOP_SMEM;
+    volatile LoopState* st = LOOP_AT(LoopState, S::O_STATE);
+    loop_begin<S>(q);
+    uint64_t a[RREG][S::CP];
+    const int lane_row = threadIdx.x / TC;
+    reg_load_rows<S>(q, st->i0, st->nrows, lane_row, threadIdx.x - lane_row * TC, a, LOOP_AT(float, S::O_A));
+    __syncthreads();
+    int it = 0;
+    while (true) {
+        ++it;
+        if (blockIdx.x < S::NP && threadIdx.x < 32) loop_ustep<S>(q, it);
+        loop_pass_reg<S>(q, it, a);
+        __syncthreads();
+        loop_arrive<S>(q, it);
         if (__syncthreads_or(st->gave_up)) break;
         const int end = st->end;
         if (blockIdx.x < S::NP) loop_gather<S>(q);
@@ -915,6 +987,77 @@ static cudaError_t launch_loop_t(int grid, const LoopArgs& a, cudaStream_t s)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_loop<NN, PREC, TC, VW, V, RL, RB, RP, NPC>, a);
+}
+
+// ---------------------------------------------------------------------------
+// Shapes with every row on chip: n -> (rows per block aimed at, TC, V, RL, RREG).  Fewer threads
+// with more columns each leave the registers for A (8 rows of 16 columns at n = 64).  Measured
+// at n = 64, m = 1229: 256 x 16 columns 9.7 us, 512 x 8 9.6; n = 48: 288 x 8 8.0, 139 blocks of 5
+// rows instead of 87 9.0; n = 32: 39 blocks of 8 rows 7.3, 20 of 16 8.1.
+// ---------------------------------------------------------------------------
+#define TVCS_REG_TABLE(X)     \
+    X(16, 32, 64, 1, 4, 8)    \
+    X(32, 8, 256, 1, 1, 8)    \
+    X(48, 8, 288, 2, 1, 8)    \
+    X(64, 8, 256, 4, 1, 8)
+
+template <int NN, int TC, int V, int RL, int RREG>
+static bool reg_configure_t()
+{
+    using S = RegShape<NN, TC, V, RL, RREG>;
+    auto kernel = k_loop_reg<NN, TC, V, RL, RREG>;
+    int per = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(S::RMAX)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, S::THREADS, S::smem(S::RMAX)) != cudaSuccess ||
+        per < 1) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
+bool reg_configure(int n)
+{
+#define X(NN, MR, TC, V, RL, RREG) \
+    if (n == NN) return reg_configure_t<NN, TC, V, RL, RREG>();
+    TVCS_REG_TABLE(X)
+#undef X
+    return false;
+}
+
+int reg_grid(int n, int m, int num_sms)
+{
+    if (num_sms < n / 2) return 0;
+#define X(NN, MR, TC, V, RL, RREG)                                              \
+    if (n == NN) {                                                              \
+        const int g = std::min(num_sms, std::max(n / 2, (m + MR - 1) / MR));    \
+        return (m + g - 1) / g <= RegShape<NN, TC, V, RL, RREG>::RMAX ? g : 0;  \
+    }
+    TVCS_REG_TABLE(X)
+#undef X
+    return 0;
+}
+
+cudaError_t launch_loop_reg(int n, int grid, const LoopArgs& a, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // the blocks wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+#define X(NN, MR, TC, V, RL, RREG)                                                    \
+    if (n == NN) {                                                                    \
+        using S = RegShape<NN, TC, V, RL, RREG>;                                      \
+        cfg.blockDim = dim3(S::THREADS, 1, 1);                                        \
+        cfg.dynamicSmemBytes = S::smem((a.m + grid - 1) / grid);                      \
+        return cudaLaunchKernelEx(&cfg, k_loop_reg<NN, TC, V, RL, RREG>, a);          \
+    }
+    TVCS_REG_TABLE(X)
+#undef X
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_loop(int prec, int n, int grid, const LoopArgs& a, cudaStream_t s)

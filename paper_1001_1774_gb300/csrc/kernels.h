@@ -105,7 +105,7 @@ struct LoopArgs {
     const unsigned char* P0;
     const unsigned char* P1;
     const float* rscale;
-    int m;
+    int prec, m;
     const float* y;           // data f
     float *u, *w, *lam, *g, *r;   // the handle's state arrays
     const float2* tw;
@@ -125,6 +125,30 @@ struct LoopArgs {
 bool loop_configure(int prec, int n);
 int loop_grid(int prec, int n, int m, int num_sms);
 cudaError_t launch_loop(int prec, int n, int grid, const LoopArgs& a, cudaStream_t s);
+
+// The same loop for n <= 64 where every row of A fits on chip.
+bool reg_configure(int n);
+int reg_grid(int n, int m, int num_sms);     // blocks of the launch, 0 where the rows do not fit
+cudaError_t launch_loop_reg(int n, int grid, const LoopArgs& a, cudaStream_t s);
+
+// The power iteration of such a handle as one launch (k_power.cu): `iters` rounds from v = v0 in
+// every entry, then ctrl->r2 = ||A v||^2.
+struct PowerArgs {
+    const unsigned char* P0;
+    const unsigned char* P1;
+    const float* rscale;
+    int prec, m, iters, one_max;
+    float v0;
+    uint64_t* xbuf;           // power_words words, zeroed once; tags as in LoopArgs
+    uint32_t tag0;
+    float2* r2part;           // grid
+    Ctrl* ctrl;
+    long long budget;
+};
+bool power_configure(int n);
+int power_grid(int n, int m, int num_sms);   // blocks of the launch, 0 where the rows do not fit
+size_t power_words(int n, int grid);
+cudaError_t launch_power(int n, int grid, PowerArgs a, cudaStream_t s);
 
 // The same products for n = 192 and 256 (binary32, bf16 hi+lo, or fp8 e4m3 + bf16
 // correction): clusters of CS blocks split each row's columns.

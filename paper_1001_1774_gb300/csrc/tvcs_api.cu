@@ -56,6 +56,7 @@ tvcs_status fail(tvcs_status s, const char* fmt, ...)
 std::mutex g_cfg_mutex;
 std::set<std::tuple<int, int, int>> g_configured;  // (device, precision, n) with the product kernel configured
 std::set<std::tuple<int, int, int>> g_loop_configured;   // and the loop kernel
+std::set<std::pair<int, int>> g_reg_configured;        // device, n: the loop and power kernels with A on chip
 
 }  // namespace
 
@@ -351,6 +352,7 @@ tvcs_status launch_iterations(tvcs_ctx* h, int iters)
     a.P0 = h->A ? reinterpret_cast<const unsigned char*>(h->A) : h->P0;
     a.P1 = h->P1;
     a.rscale = h->rscale;
+    a.prec = h->opt.precision;
     a.m = h->m;
     a.y = h->f;
     a.u = h->u;
@@ -375,7 +377,10 @@ tvcs_status launch_iterations(tvcs_ctx* h, int iters)
     h->loop_tag += (uint32_t)iters;
     a.budget = budget_of(h);
     a.bar_extra = h->bar_extra;
-    CK(launch_loop(h->opt.precision, h->n, h->loop_grid, a, h->stream));
+    if (h->loop_reg)
+        CK(launch_loop_reg(h->n, h->loop_grid, a, h->stream));
+    else
+        CK(launch_loop(h->opt.precision, h->n, h->loop_grid, a, h->stream));
     return TVCS_OK;
 }
 
@@ -433,10 +438,41 @@ tvcs_status run_loop(tvcs_ctx* h, int iters, double tol, tvcs_result* res)
     return st;
 }
 
+// tau from ||A v||^2 of the power iteration's last v.
+tvcs_status tau_of(tvcs_ctx* h, double* tau_out)
+{
+    const double lmax = h->hctrl->r2;
+    if (!(lmax > 0.0) || !isfinite(lmax))
+        return fail(TVCS_ERR_DIVERGED, "power iteration gave lambda_max = %g", lmax);
+    *tau_out = 1.0 / (1.01 * lmax);
+    return TVCS_OK;
+}
+
 tvcs_status power_tau(tvcs_ctx* h, int iters, double* tau_out)
 {
     const int N = h->N;
-    launch_fill(h->tx, N, (float)(1.0 / sqrt((double)N)), h->stream);
+    const float v0 = (float)(1.0 / sqrt((double)N));
+    if (h->power_grid) {   // all rounds in one launch
+        PowerArgs a{};
+        a.P0 = h->A ? reinterpret_cast<const unsigned char*>(h->A) : h->P0;
+        a.P1 = h->P1;
+        a.rscale = h->rscale;
+        a.prec = h->opt.precision;
+        a.m = h->m;
+        a.iters = iters;
+        a.v0 = v0;
+        a.xbuf = h->ubuf;
+        a.tag0 = h->loop_tag;
+        h->loop_tag += (uint32_t)iters;
+        a.r2part = h->r2part;
+        a.ctrl = h->ctrl;
+        a.budget = budget_of(h);
+        CK(launch_power(h->n, h->power_grid, a, h->stream));
+        CKS(read_ctrl(h));
+        if (h->hctrl->error == ERR_TIMEOUT) return fail(TVCS_ERR_TIMEOUT, "a bounded device wait gave up");
+        return tau_of(h, tau_out);
+    }
+    launch_fill(h->tx, N, v0, h->stream);
     for (int it = 0; it < iters; ++it) {
         products(h, h->tx, nullptr, h->tr, h->gpart2, nullptr, MODE_PLAIN, 0ull, 0, h->stream);
         launch_gather(h->gpart2, h->P, N, 1.0f, h->tg, h->part, h->ctrl, h->stream);
@@ -444,11 +480,7 @@ tvcs_status power_tau(tvcs_ctx* h, int iters, double* tau_out)
     }
     products(h, h->tx, nullptr, h->tr, h->gpart2, nullptr, MODE_PLAIN, 0ull, 0, h->stream);
     CKS(read_ctrl(h));
-    const double lmax = h->hctrl->r2;
-    if (!(lmax > 0.0) || !isfinite(lmax))
-        return fail(TVCS_ERR_DIVERGED, "power iteration gave lambda_max = %g", lmax);
-    *tau_out = 1.0 / (1.01 * lmax);
-    return TVCS_OK;
+    return tau_of(h, tau_out);
 }
 
 tvcs_status check_handle(tvcs_handle h)
@@ -517,7 +549,7 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
 {
     CK(cudaGetDevice(&h->dev));
     CK(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->dev));
-    bool loop_ok = false;
+    bool loop_ok = false, reg_ok = false;
     {
         std::lock_guard<std::mutex> lk(g_cfg_mutex);
         const int prec = h->opt.precision;
@@ -527,6 +559,9 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
             if (loop_configure(prec, h->n)) g_loop_configured.insert({h->dev, prec, h->n});
         }
         loop_ok = g_loop_configured.count({h->dev, prec, h->n}) != 0;
+        if (!g_reg_configured.count({h->dev, h->n}) && reg_configure(h->n) && power_configure(h->n))
+            g_reg_configured.insert({h->dev, h->n});
+        reg_ok = g_reg_configured.count({h->dev, h->n}) != 0;
     }
     if (h->opt.stream) {
         h->stream = (cudaStream_t)h->opt.stream;
@@ -555,8 +590,13 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     h->ucluster = usolve_choose_cluster(h->n);
     if (h->ucluster == 0)
         return fail(TVCS_ERR_UNSUPPORTED, "no thread-block cluster of 8 or 16 fits for n = %d", h->n);
-    if (!noA && loop_ok) h->loop_grid = loop_grid(prec, h->n, h->m, h->num_sms);
-    const size_t P = (size_t)std::max(h->P, h->loop_grid);   // partials of A^T r
+    if (!noA && reg_ok) {
+        h->loop_grid = reg_grid(h->n, h->m, h->num_sms);
+        h->loop_reg = h->loop_grid > 0;
+        if (!(h->opt.tau > 0.0)) h->power_grid = power_grid(h->n, h->m, h->num_sms);
+    }
+    if (!noA && loop_ok && !h->loop_reg) h->loop_grid = loop_grid(prec, h->n, h->m, h->num_sms);
+    const size_t P = (size_t)std::max(h->P, std::max(h->loop_grid, h->power_grid));   // partials of A^T r and ||r||^2
     const size_t nparts = 2 * (size_t)((N + 255) / 256 + 1024);
     // A: binary32 for the classic path and as the source of the split storages.
     if (!noA) CKS(alloc((void**)&h->A, sizeof(float) * m * N));
@@ -578,9 +618,11 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     CKS(alloc((void**)&h->gpart, sizeof(float) * N * P));
     CKS(alloc((void**)&h->gpart2, sizeof(float) * N * (size_t)h->P));
     CKS(alloc((void**)&h->r2part, sizeof(float2) * P));
-    if (h->loop_grid) {
-        // ubuf, colx, rowx of 2 N words and nbuf of 4 n, in one zeroed array
-        const size_t words = 6 * N + 4 * (size_t)h->n;
+    if (h->loop_grid || h->power_grid) {
+        // ubuf, colx, rowx of 2 N words and nbuf of 4 n (k_loop.cu), or what k_power.cu wants,
+        // in one zeroed array
+        size_t words = h->loop_grid ? 6 * N + 4 * (size_t)h->n : 0;
+        if (h->power_grid) words = std::max(words, power_words(h->n, h->power_grid));
         CKS(alloc((void**)&h->ubuf, sizeof(uint64_t) * words));
         CK(cudaMemsetAsync(h->ubuf, 0, sizeof(uint64_t) * words, h->stream));
         h->colx = h->ubuf + 2 * N;

@@ -121,3 +121,24 @@ def test_dct_loop_against_the_oracle_and_the_single_launches(tv, n, m, algo, ite
     if tol == 0.0:
         for a, b in zip(*out):
             assert rel(a, b) <= 3e-5 or np.linalg.norm(b) == 0.0
+
+
+# A on chip (n <= 64): fewer rows than blocks, a row more or less than the registers hold, rows in
+# shared memory, and (64, 3500), whose rows do not fit; tau from the power iteration.  The power
+# iteration's ||A v||^2 carries about 4 roundings of 2^-24 of every dot product, taken as
+# independent over N: well below 1e-5; the two runs then agree as above.
+@pytest.mark.parametrize("n,m,prec", [
+    (16, 1, 0), (16, 31, 0), (16, 256, 0), (32, 15, 0), (32, 128, 1), (32, 129, 0), (32, 1024, 2), (48, 24, 0),
+    (48, 1217, 0), (48, 2304, 0), (64, 31, 0), (64, 257, 2), (64, 1216, 0), (64, 1230, 1), (64, 2600, 0), (64, 3500, 0)])
+def test_rows_on_chip_and_the_power_iteration(tv, n, m, prec):
+    P = synth.make_problem(n, 0.0, 3, 4, 1e3, 10.0, m=m, noise_c=1e-3)
+    A = np.ascontiguousarray(quant_ref.effective_A(P.A, prec))
+    tau = oracle.default_tau(A)
+    h = create(tv, P, 0.0, prec, 0, 8)
+    assert abs(tv.tvcs_get_tau(h) / tau - 1) <= 1e-5
+    k = create(tv, P, tv.tvcs_get_tau(h), prec, 0, 8, host_loop=1)
+    u, v = np.empty(n * n, np.float32), np.empty(n * n, np.float32)
+    a, b = tv.tvcs_solve(h, P.f, u), tv.tvcs_solve(k, P.f, v)
+    assert a.iters == b.iters == 8 and rel(u, v) <= 1e-5
+    r = tv.get_state(h, tv.TVCS_STATE_R).astype(np.float64)
+    assert abs(a.resid2 - (r * r).sum()) <= 1e-9 * a.resid2
