@@ -85,100 +85,146 @@ void launch_batch_cond(const Ctrl* ctrls, int count, Ctrl* bctrl, unsigned long 
 // three-level sum: 32 products from zero, 16 such chunks, then the running total
 // (the tensor-core products keep 16 bits of u and add in one long binary32 chain,
 // which is accurate for the iteration but not for ||r||^2 of a converged image).
-// Block: 64 rows x 64 images, 256 threads of 4 x 4 outputs; K in chunks of 32.
-constexpr int RS_BM = 64, RS_BB = 64, RS_BK = 32;
+//
+// Block: 4 warps of 6 rows x 32 IPL images, K in chunks of 32, double-buffered.  A lane has IPL
+// images (lane, lane + 32, ..); rows go in pairs through packed FMAs.  A chunk of U lies as it
+// is in memory (one 16-byte load gives a lane 4 columns of an image, images 36 floats apart: no
+// bank conflicts), a chunk of A transposed, so that a row pair is one operand and all lanes
+// read the same words.  The order of every output's sum is the one above, whatever the split.
+//
+// What bounds it: FMA issue (4915 x 16384 x 256: 0.56 ms at 128 FMAs a cycle and SM) and how
+// blocks divide over the SMs.  Measured there with 4, 6, 8 rows a warp: 1.37, 1.05, 1.27 ms (8
+// rows: 308 blocks, 2.03 an SM, so that some have 3; 4 rows: as many shared-memory as FMA
+// cycles), 512 images 2.34, 2.00, 2.06.  64 x 64 blocks of 4 x 4 outputs a thread,
+// single-buffered, took 1.98 and 4.00 ms.
+constexpr int RS_RP = 3, RS_BM = 4 * 2 * RS_RP, RS_BK = 32, RS_UP = RS_BK + 4, RS_AP = 4 * 8 + 4;   // RS_RP row pairs a warp
 
-__global__ void __launch_bounds__(256)
+template <int IPL>
+__global__ void __launch_bounds__(128)
     k_batch_resid(const unsigned short* __restrict__ hi, const unsigned short* __restrict__ lo,
                   int m, int N, const float* __restrict__ U, const float* __restrict__ F,
                   int count, float* __restrict__ R)
 {
-    __shared__ float As[RS_BK][RS_BM + 4];
-    __shared__ float Us[RS_BK][RS_BB + 4];
-    const int tid = threadIdx.x;
-    const int tx = tid & 15, ty = tid >> 4;              // images tx*4.., rows ty*4..
-    const int i0 = blockIdx.x * RS_BM, b0 = blockIdx.y * RS_BB;
-    float c[4][4], l1[4][4], l2[4][4];
+    constexpr int BB = 32 * IPL;
+    __shared__ __align__(16) float Us[2][BB][RS_UP];
+    __shared__ __align__(16) float As[2][RS_BK][RS_AP];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = blockIdx.x * RS_BM, b0 = blockIdx.y * BB;
+    uint64_t l1[RS_RP][IPL], l2[RS_RP][IPL];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int p = 0; p < RS_RP; ++p)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) l1[a][b] = l2[a][b] = 0.f;
-    const int lr = tid >> 2, lg = (tid & 3) * 8;         // loader: row / image lr, columns lg..lg+7
-    int chunk = 0;
-    for (int k0 = 0; k0 < N; k0 += RS_BK, ++chunk) {
-        {   // A_eff tile (transposed) and U tile (transposed)
-            const int i = i0 + lr;
-            float av[8];
-            if (i < m) {
-                const uint4 h = *reinterpret_cast<const uint4*>(hi + (size_t)i * N + k0 + lg);
-                const uint4 l = *reinterpret_cast<const uint4*>(lo + (size_t)i * N + k0 + lg);
-                const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+        for (int q = 0; q < IPL; ++q) l1[p][q] = l2[p][q] = 0ull;
+    const int lr = tid >> 2, lg = (tid & 3) * 8;   // A's loader: row lr, columns lg .. lg + 7
+    uint4 ah = make_uint4(0u, 0u, 0u, 0u), al = ah;
+    auto load_a = [&](int k0) {
+        if (lr < RS_BM && i0 + lr < m) {
+            ah = *reinterpret_cast<const uint4*>(hi + (size_t)(i0 + lr) * N + k0 + lg);
+            al = *reinterpret_cast<const uint4*>(lo + (size_t)(i0 + lr) * N + k0 + lg);
+        }
+    };
+    const int as = lr / (2 * RS_RP) * 8 + lr % (2 * RS_RP);   // a warp's rows from a multiple of 8
+    auto store_a = [&](int buf) {
+        if (lr >= RS_BM) return;
+        const uint32_t hw[4] = {ah.x, ah.y, ah.z, ah.w}, lw[4] = {al.x, al.y, al.z, al.w};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    av[2 * q] = __uint_as_float(hw[q] << 16) + __uint_as_float(lw[q] << 16);
-                    av[2 * q + 1] = __uint_as_float(hw[q] & 0xffff0000u) +
-                                    __uint_as_float(lw[q] & 0xffff0000u);
-                }
-            } else {
+        for (int q = 0; q < 4; ++q) {
+            As[buf][lg + 2 * q][as] = __uint_as_float(hw[q] << 16) + __uint_as_float(lw[q] << 16);
+            As[buf][lg + 2 * q + 1][as] =
+                __uint_as_float(hw[q] & 0xffff0000u) + __uint_as_float(lw[q] & 0xffff0000u);
+        }
+    };
+    const int ub = tid >> 3, uc = 4 * (tid & 7);   // U's loader: images ub, ub + 16, .., columns uc ..
+    const float* usrc = U + (size_t)(b0 + ub) * N + uc;
+    auto load_u = [&](int buf, int k0) {   // images past the last: zeros
 #pragma unroll
-                for (int q = 0; q < 8; ++q) av[q] = 0.f;
+        for (int e = 0; e < 2 * IPL; ++e) {
+            const bool there = b0 + ub + 16 * e < count;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(&Us[buf][ub + 16 * e][uc])),
+                         "l"(there ? usrc + (size_t)16 * e * N + k0 : U), "r"(there ? 16 : 0)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    load_u(0, 0);
+    load_a(0);
+    store_a(0);
+    const int chunks = N / RS_BK;
+    for (int ch = 0; ch < chunks; ++ch) {
+        const int buf = ch & 1;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // this chunk is there, and nobody reads the other buffer any more
+        if (ch + 1 < chunks) {
+            load_u(buf ^ 1, (ch + 1) * RS_BK);
+            load_a((ch + 1) * RS_BK);
+        }
+        uint64_t c[RS_RP][IPL];
+#pragma unroll
+        for (int p = 0; p < RS_RP; ++p)
+#pragma unroll
+            for (int q = 0; q < IPL; ++q) c[p][q] = 0ull;
+#pragma unroll
+        for (int k4 = 0; k4 < RS_BK; k4 += 4) {
+            float u[IPL][4];
+#pragma unroll
+            for (int q = 0; q < IPL; ++q) {
+                const float4 t = *reinterpret_cast<const float4*>(&Us[buf][lane + 32 * q][k4]);
+                u[q][0] = t.x; u[q][1] = t.y; u[q][2] = t.z; u[q][3] = t.w;
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) As[lg + q][lr] = av[q];
-            const int b = b0 + lr;
-            float uv[8];
-            if (b < count) {
-                const float4 u0 = *reinterpret_cast<const float4*>(U + (size_t)b * N + k0 + lg);
-                const float4 u1 = *reinterpret_cast<const float4*>(U + (size_t)b * N + k0 + lg + 4);
-                uv[0] = u0.x; uv[1] = u0.y; uv[2] = u0.z; uv[3] = u0.w;
-                uv[4] = u1.x; uv[5] = u1.y; uv[6] = u1.z; uv[7] = u1.w;
-            } else {
+            for (int k = 0; k < 4; ++k) {
+                const ulonglong2* ap = reinterpret_cast<const ulonglong2*>(&As[buf][k4 + k][warp * 8]);
+                const ulonglong2 a0 = ap[0], a1 = ap[1];
+                const uint64_t a[4] = {a0.x, a0.y, a1.x, a1.y};
 #pragma unroll
-                for (int q = 0; q < 8; ++q) uv[q] = 0.f;
+                for (int q = 0; q < IPL; ++q) {
+                    const uint64_t uu = pack2(u[q][k], u[q][k]);
+#pragma unroll
+                    for (int p = 0; p < RS_RP; ++p) c[p][q] = fma2(a[p], uu, c[p][q]);
+                }
             }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) Us[lg + q][lr] = uv[q];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) c[a][b] = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < RS_BK; ++k) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 u4 = *reinterpret_cast<const float4*>(&Us[k][tx * 4]);
-            const float av[4] = {a4.x, a4.y, a4.z, a4.w}, uv[4] = {u4.x, u4.y, u4.z, u4.w};
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) c[a][b] = fmaf(av[a], uv[b], c[a][b]);
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int p = 0; p < RS_RP; ++p)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) l1[a][b] += c[a][b];
-        if ((chunk & 15) == 15) {
+            for (int q = 0; q < IPL; ++q) l1[p][q] = add2(l1[p][q], c[p][q]);
+        if ((ch & 15) == 15) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int p = 0; p < RS_RP; ++p)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    l2[a][b] += l1[a][b];
-                    l1[a][b] = 0.f;
+                for (int q = 0; q < IPL; ++q) {
+                    l2[p][q] = add2(l2[p][q], l1[p][q]);
+                    l1[p][q] = 0ull;
                 }
         }
-        __syncthreads();
+        if (ch + 1 < chunks) store_a(buf ^ 1);
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int i = i0 + ty * 4 + a;
-        if (i >= m) continue;
+    for (int q = 0; q < IPL; ++q) {
+        const int img = b0 + lane + 32 * q;
+        if (img >= count) continue;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int img = b0 + tx * 4 + b;
-            if (img < count) R[(size_t)img * m + i] = (l2[a][b] + l1[a][b]) - F[(size_t)img * m + i];
+        for (int p = 0; p < RS_RP; ++p) {
+            const float2 t = unpack2(add2(l2[p][q], l1[p][q]));
+            const int i = i0 + warp * 2 * RS_RP + 2 * p;
+            const size_t o = (size_t)img * m + i;
+            if (i < m) R[o] = t.x - F[o];
+            if (i + 1 < m) R[o + 1] = t.y - F[o + 1];
         }
     }
+}
+
+static void launch_batch_resid(const unsigned short* hi, const unsigned short* lo, int m, int N, const float* U,
+                        const float* F, int count, float* R, cudaStream_t s)
+{
+    // fewer images a lane where the others would be padding (each costs its FMAs)
+    const int rows = (m + RS_BM - 1) / RS_BM;
+    if (count > 64)
+        k_batch_resid<4><<<dim3(rows, (count + 127) / 128), 128, 0, s>>>(hi, lo, m, N, U, F, count, R);
+    else if (count > 32)
+        k_batch_resid<2><<<dim3(rows, 1), 128, 0, s>>>(hi, lo, m, N, U, F, count, R);
+    else
+        k_batch_resid<1><<<dim3(rows, 1), 128, 0, s>>>(hi, lo, m, N, U, F, count, R);
 }
 
 // ctrls[b].r2 = ||R_b||^2 (double-single, fixed order), one block per image.
@@ -809,9 +855,8 @@ tvcs_status solve_batch(tvcs_ctx* h, int count, const float* const* f, float* co
     }
     // end of run, per image: ||r||^2 of the image's own residual recomputed on the CUDA
     // cores, final multiplier update, objective, residuals
-    k_batch_resid<<<dim3((h->m + RS_BM - 1) / RS_BM, (count + RS_BB - 1) / RS_BB), 256, 0, s>>>(
-        reinterpret_cast<const unsigned short*>(h->P0), reinterpret_cast<const unsigned short*>(h->P1),
-        h->m, h->N, b->U, b->F, count, b->R);
+    launch_batch_resid(reinterpret_cast<const unsigned short*>(h->P0), reinterpret_cast<const unsigned short*>(h->P1),
+                       h->m, h->N, b->U, b->F, count, b->R, s);
     k_batch_resid_r2<<<count, 256, 0, s>>>(b->R, h->m, b->ctrls);
     TvArgs a = batch_tv_args(h, count, MODE_PLAIN);
     launch_tv(h->n, a, 4, s);

@@ -547,3 +547,33 @@ def test_batched_n128_u_solve_in_registers(tv):
     assert rel(us[2], u1) <= 1e-4
     tv.tvcs_destroy(h)
     tv.tvcs_destroy(h1)
+
+
+# The end-of-run residual of a batch (24 rows and 32, 64 or 128 images a block) against the
+# same three-level binary32 sum on the host: the same bits, at rows and images that fill no block.
+@pytest.mark.parametrize("m,count", [(1, 1), (23, 33), (25, 31), (131, 64), (47, 129), (24, 65)])
+def test_end_residual_has_the_bits_of_its_sum(tv, m, count):
+    n, N = 32, 1024
+    rng = np.random.default_rng(m + count)
+    A = (rng.standard_normal((m, N)) / np.sqrt(N)).astype(np.float32)
+    opt = tv.tvcs_default_options()
+    opt.tau, opt.max_iter, opt.precision = 0.1, 2, 1
+    h = tv.tvcs_create(torch.from_numpy(A).cuda(), 0, m, n, 10.0, 10.0, 0.0, opt)
+    F = torch.from_numpy(rng.standard_normal((count, m)).astype(np.float32)).cuda()
+    U = torch.empty(count, N, device="cuda")
+    res = tv.tvcs_solve_batched([h] * count, list(F), list(U))
+    u, f = U.cpu().numpy().astype(np.float64), F.cpu().numpy()
+    a = quant_ref.effective_A(A, 1).astype(np.float64)
+    l1 = np.zeros((count, m), np.float32)
+    l2 = np.zeros((count, m), np.float32)
+    for ch in range(N // 32):
+        c = np.zeros((count, m), np.float32)
+        for k in range(32 * ch, 32 * ch + 32):   # an FMA: exact in binary64 up to one rare double rounding
+            c = (u[:, k, None] * a[None, :, k] + c).astype(np.float32)
+        l1 = l1 + c
+        if ch % 16 == 15:
+            l2, l1 = l2 + l1, np.zeros_like(l1)
+    r = ((l2 + l1) - f).astype(np.float64)
+    for b in range(count):
+        # one ulp of the odd double rounding in one partial sum; else equal to the sums' 44 bits
+        assert abs(res[b].resid2 - (r[b] ** 2).sum()) <= 1e-7 * res[b].resid2
