@@ -225,7 +225,7 @@ def traffic_from_profile(summary=PROFILE_SUMMARY, key="dram_bytes_per_launch"):
 
 
 def batch_launch_iters(iters):
-    """The same for the shared-A batch, whose loop body holds 4 iterations."""
+    """The same for the batches (shared A, uneven), whose loop bodies hold 4 iterations."""
     return -(-iters // 4) * 4
 
 
@@ -256,6 +256,15 @@ def loop_launch_iters(iters, max_iter=None):
     if iters <= nb * body:
         return -(-iters // body) * body + rest
     return max_iter
+
+
+def loop_launches(n, iters, max_iter=None, dct=False, host_loop=False):
+    """Kernels of a single-image run's iterations: one persistent launch for the
+    partial-DCT encoder and for a stored A up to 96 x 96, else the u-solve and the
+    products of every launched iteration."""
+    if (dct or n <= 96) and not host_loop:
+        return 1
+    return 2 * loop_launch_iters(iters, max_iter)
 
 
 # ----------------------------------------------------------------------------- CPU oracle sample
@@ -428,7 +437,7 @@ def run_ours(args):
                     "d2h_bytes_per_step": 4 * P.N / ITERS_PER_RECON,
                     "note": "tvcs_solve with pinned host f and u, %d reconstructions of %d iterations"
                             % (args.e2e_solves, ITERS_PER_RECON)},
-            "gpu_launches": 2 * loop_launch_iters(args.steps) + 2,
+            "gpu_launches": loop_launches(P.n, args.steps, host_loop=args.host_loop) + 2,
             "clocks": clocks,
             "tau": tau,
             "relative_error_vs_phantom": rel_err_ubar,
@@ -785,7 +794,7 @@ def run_uneven(args):
            "e2e": {"value": sum(r.iters for r in res_e) / e2e_s, "unit": "problem-iter/s",
                    "h2d_bytes_per_step": 4 * sum(P.m for P in probs) / loops,
                    "d2h_bytes_per_step": 4 * sum(P.N for P in probs) / loops},
-           "gpu_launches": (len({P.n for P in probs}) + 3) * loops + 6,
+           "gpu_launches": (len({P.n for P in probs}) + 3) * batch_launch_iters(loops) + 6,
            "setup_seconds": {"inputs": t_gen, "create_64_handles": t_create, "warmup_solve": t_warm},
            "clocks": clocks}
     if not args.no_cpu_baseline:
@@ -893,14 +902,16 @@ def run_dct(args):
                         "peak": fp32_peak, "unit": "TFLOP/s",
                         "frac": flops / (prod_us * 1e-6) / 1e12 / fp32_peak, "traffic": None,
                         "kernel": "k_dct_products (one 16-block cluster)",
-                        "note": "latency-bound: 16.8 MFLOP per launch on one 16-SM cluster "
-                                "(the peak is the whole GPU's; the cluster's 16 SMs have 8.5 TFLOP/s)",
+                        "note": "a launch of the products alone, as tvcs_apply runs them (16.8 MFLOP on one "
+                                "16-SM cluster: the peak is the whole GPU's, the cluster's 16 SMs have 8.5 "
+                                "TFLOP/s); the loop is one launch of k_dct_loop with FFTs, %.2f us an "
+                                "iteration" % (ms * 1e3 / iters),
                         "launch_us": prod_us,
                         "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 FLOP x 2070 MHz"},
            "stage_us": {"dct_products": prod_us, "usolve_cluster": us_us},
            "e2e": {"value": r_e.iters / e2e_s, "unit": "iter/s",
                    "h2d_bytes_per_step": 4 * P.m / r_e.iters, "d2h_bytes_per_step": 4 * P.N / r_e.iters},
-           "gpu_launches": nrec * (2 * loop_launch_iters(res.iters, P.max_iter) + 2),
+           "gpu_launches": nrec * (loop_launches(n, res.iters, P.max_iter, dct=True) + 2),
            "relative_error_vs_phantom": float(np.linalg.norm(u_gpu - ub) / np.linalg.norm(ub)),
            "clocks": clocks}
     if not args.no_cpu_baseline:

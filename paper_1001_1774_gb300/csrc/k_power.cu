@@ -5,13 +5,14 @@
 // binary32: RL RREG of them in registers, the rest in shared memory.  Every block keeps the whole
 // v, so that only A^T r travels, as the words of loop_exchange.cuh: with few blocks every block
 // adds all partials, else the owner of a slice of SL columns adds its partials and sends the
-// sums to all.  A buffer is written again only after every block has sent something that it could
+// sums to all, with its part of ||g||^2 (binary64 runs at 1/64 of the binary32 rate here: every
+// block squaring all of g took 2 of 10 us a round at 64 x 64).  A buffer is written again only after every block has sent something that it could
 // not have sent before reading the buffer.
 //
 // What bounds it: latency (one or two exchanges of about 1.2 us and six block barriers a round;
 // the products are 0.5 us).  A launch of the products, one of the partials' sum and one of the
 // scaling took about 20 us a round at every size; tvcs_create with 100 rounds: 16 x 16 (m = 77)
-// 1.87 -> 0.49 ms, 32 x 32 (307) 2.49 -> 0.97, 48 x 48 (691) 2.74 -> 1.20, 64 x 64 (1229) 3.12 -> 1.62.
+// 1.87 -> 0.49 ms, 32 x 32 (307) 2.49 -> 0.93, 48 x 48 (691) 2.74 -> 1.08, 64 x 64 (1229) 3.12 -> 1.44.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -74,17 +75,15 @@ __device__ __forceinline__ void power_inverse_norm(PowerState* st, double s)
     st->lo = (float)(f - (double)st->hi);
 }
 
-// v <- v / ||v||; the norm in binary64, as its square may be out
-// of binary32's range.
+// v <- v / ||v||, the sum of the threads' s being ||v||^2 in binary64 (it may be out of binary32's
+// range).
 template <class S>
-__device__ __forceinline__ void power_normalize()
+__device__ __forceinline__ void power_normalize(double s)
 {
     POWER_SMEM;
     const int tid = fresh_tid();
     PowerState* st = POWER_AT(PowerState, S::O_STATE);
     float* sv = POWER_AT(float, S::O_V);
-    double s = 0.0;
-    for (int i = tid; i < S::N; i += S::THREADS) s = fma((double)sv[i], (double)sv[i], s);
     s = block_sum(s, POWER_AT(double, S::O_DRED));
     if (tid == 0) power_inverse_norm(st, s);
     __syncthreads();
@@ -132,7 +131,9 @@ __global__ void __launch_bounds__(TC * RL, 1) k_power(const __grid_constant__ Po
 
         // the partial, two exchanges: [slice][block][SL], one: [round & 1][block][N]
         uint64_t* part = q.xbuf + (two ? 0 : (size_t)(it & 1) * G * N);
-        uint64_t* sums = q.xbuf + (size_t)G * N;   // two exchanges
+        uint64_t* sums = q.xbuf + (size_t)G * N;   // two exchanges: the sums, then every slice's part of ||g||^2
+        uint64_t* norms = sums + N;
+        double sq = 0.0;
         auto send_partial = [&](int c, uint64_t pair) {
             const float2 t = unpack2(pair);
             send2(two ? part + ((size_t)(c / SL) * G + blk) * SL + c % SL : part + (size_t)blk * N + c, t.x, t.y, tag);
@@ -190,6 +191,11 @@ __global__ void __launch_bounds__(TC * RL, 1) k_power(const __grid_constant__ Po
                     z.x += __shfl_xor_sync(0xffffffffu, z.x, 16);
                     z.y += __shfl_xor_sync(0xffffffffu, z.y, 16);
                     if (h == 0) send2(sums + (size_t)s * SL + 2 * c, z.x, z.y, tag);
+                    double d = fma((double)z.y, (double)z.y, (double)z.x * (double)z.x);
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                    if (lane == 0)
+                        send2(norms + 2 * s, __int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)), tag);
                 }
             }
             constexpr int K = (N / 2 + T - 1) / T;
@@ -199,6 +205,12 @@ __global__ void __launch_bounds__(TC * RL, 1) k_power(const __grid_constant__ Po
 #pragma unroll
             for (int k = 0; k < K; ++k)
                 if (k < n) reinterpret_cast<float2*>(sv)[tid + k * T] = make_float2(word_f(v[k].x), word_f(v[k].y));
+            static_assert(N / SL <= T, "a slice's norm a thread");
+            if (tid < N / SL) {
+                ulonglong2 d[1];
+                poll2<1>(d, 1, tag, waits, [&](int) { return norms + 2 * tid; });
+                sq = __hiloint2double((int)(uint32_t)d[0].y, (int)(uint32_t)d[0].x);
+            }
         } else if (G > 1) {
 #pragma unroll 1
             for (int i = tid; i < N / 2; i += T) {
@@ -224,7 +236,9 @@ __global__ void __launch_bounds__(TC * RL, 1) k_power(const __grid_constant__ Po
         }
         // (the vote makes the outcome the same for every thread of the block)
         if (__syncthreads_or(st->gave_up)) break;
-        power_normalize<S>();
+        if (!two)
+            for (int i = tid; i < N; i += T) sq = fma((double)sv[i], (double)sv[i], sq);
+        power_normalize<S>(sq);
     }
 
     // ||A v||^2 over the blocks, by the last one to come
