@@ -303,8 +303,14 @@ int power_grid(int n, int m, int num_sms)
 
 size_t power_words(int n, int grid)
 {
-    // one exchange: two sets of partials; two: one set and the sums
-    return (size_t)2 * grid * n * n + (size_t)n * n;
+    const size_t N = (size_t)n * n;
+    int one = 0;
+#define X(NN, TGT, ONE, TC, V, RL, RREG) \
+    if (n == NN) one = ONE;
+    TVCS_POWER_TABLE(X)
+#undef X
+    // one exchange: two sets of partials; two: one set, the sums, two words of norm a slice
+    return grid <= one ? 2 * grid * N : (grid + 1) * N + 2 * (N / 32);
 }
 
 cudaError_t launch_power(int n, int grid, PowerArgs a, cudaStream_t s)

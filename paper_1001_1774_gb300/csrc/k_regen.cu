@@ -101,7 +101,7 @@ __device__ int active_prefix(const RegenProb* __restrict__ probs, int P, int mod
 // The k-th chunk of cluster q of Q: there and back over the clusters, so that with the largest
 // chunks first (the order of the problem table) the clusters' sums stay within about a chunk of
 // each other.  (Equal contiguous shares of the entries gave some clusters a large chunk and a
-// share of small ones: six problems of 114 M entries 0.52 ms a launch, here 0.40.)
+// share of small ones: six problems of 114 M entries 0.52 ms a launch, here 0.43.)
 __device__ __forceinline__ int chunk_of(int k, int q, int Q)
 {
     return (k & 1) ? (k + 1) * Q - 1 - q : k * Q + q;

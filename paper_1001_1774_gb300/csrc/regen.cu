@@ -116,8 +116,8 @@ tvcs_status ralloc(void** p, size_t bytes)
 // Rows per chunk: about 2^21 entries of A, and at most m/16 rows so that a small
 // problem still spreads over 16 clusters; fixed by the problem alone, so that
 // the chunk slots (and with them the order of every sum of A^T r and ||r||^2)
-// do not depend on the launch shape.  (At most m/192 rows in whole tiles of 16 would be 24 %
-// faster for six problems of 114 M entries, 0.52 -> 0.40 ms, as their 2 M-entry chunks fill 39 of 72
+// do not depend on the launch shape.  (At most m/192 rows in whole tiles of 16 would be 8 %
+// faster for six problems of 114 M entries, 0.43 -> 0.40 ms, as their 2 M-entry chunks fill 39 of 72
 // clusters; it would change the order of the sums.)
 constexpr long long kChunkEntries = 1LL << 21;
 
