@@ -81,7 +81,8 @@ typedef struct {
     void* stream;        /* cudaStream_t for all device work; NULL: a stream the handle owns */
     int power_iters;     /* <= 0: 100 */
     long long timeout_cycles; /* bound of every device spin-wait, in SM clock cycles; <= 0: 2^31 */
-    int host_loop;       /* 0 (default): the iteration loop is one CUDA graph whose WHILE node
+    int host_loop;       /* 0 (default): the iteration loop is one launch (stored A up to
+                            96 x 96, partial DCT) or one CUDA graph whose WHILE node
                             the kernels end; 1: the same kernels launched from the host per
                             iteration (for profilers that cannot look inside such graphs) */
     int a_mode;          /* TVCS_A_STORED (default) or TVCS_A_REGENERATE: every product
