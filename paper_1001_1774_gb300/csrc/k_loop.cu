@@ -27,13 +27,9 @@
 // replaces (u-solve cluster, products) paid two kernel boundaries, a grid barrier with a
 // global reduction and a second read of g, and had loop graphs to build.  us an iteration, 200
 // iterations, binary32, as the chain -> k_loop -> k_loop_reg:
-//   n = 16 (m = 77) 9.6 -> 6.7 -> 4.5, n = 32 (307) 11.7 -> 7.8 -> 6.9, n = 48 (691) 12.5 -> 8.7 ->
+//   n = 16 (m = 77) 9.6 -> 6.7 -> 4.8, n = 32 (307) 11.7 -> 7.8 -> 7.3, n = 48 (691) 12.5 -> 8.7 ->
 //   8.0, n = 64 (1229) 14.75 -> 11.4 -> 9.7 (2048: 13.2 -> 10.0; fp8, 1229: 13.8 -> 9.7), n = 96
 //   (921) 17.0 -> 16.3, n = 96 (2765) 23.7 -> 23.3.
-// At n <= 32 the u-step's blocks are one cluster, and column slots and rows go through shared
-// memory instead of L2.  Through L2 an exchange costs 1 us or nearly 2, by where the buffers and
-// the blocks come to lie on the two dies: 16 x 16 4.8 or 6.1 -> 4.5 or 5.0 us an iteration,
-// 32 x 32 7.1 or 9.3 -> 6.9 or 7.3 (one device or another).
 // (From the ring a pass over 9 rows took three steps of 1.3 us, each a wait, a decode, a warp
 // reduction and a block barrier in series; from registers all rows share one of each.)  At
 // n = 128 k_loop measured 52.5 us against 52.1 (u-solve and exchanges take 13 us in which L2 cannot
@@ -83,7 +79,7 @@ template <int NN_, int PREC_, int TC_, int VW_, int V_, int RL_, int RB_, int RP
 struct LoopShape {
     using P = ProdShape<PREC_, TC_, VW_, V_, RL_, RB_, 2>;
     static_assert(P::N == NN_ * NN_, "columns");
-    static constexpr int NN = NN_, PREC = PREC_, TC = TC_, VW = VW_, V = V_, RL = RL_, RB = RB_, RREG = 0, CL = 1;
+    static constexpr int NN = NN_, PREC = PREC_, TC = TC_, VW = VW_, V = V_, RL = RL_, RB = RB_, RREG = 0;
     static constexpr int CP = P::CPT / 2;
     static constexpr int N = P::N, THREADS = P::THREADS, WARPS = P::WARPS, RS = P::RS, WPR = P::WPR;
     static constexpr int B0 = P::B0, B1 = P::B1;
@@ -121,12 +117,9 @@ struct LoopShape {
 
 // The same without a ring: every row of A on chip as binary32 for the whole launch, RL RREG of
 // them in registers (a thread has its columns of RREG rows), up to XMAX more in shared memory.
-// CL > 1: clusters of CL blocks, the first of which has all of the u-step's blocks: column slots
-// and rows then go straight to the reader's shared memory.
-template <int NN_, int TC_, int V_, int RL_, int RREG_, int CL_>
+template <int NN_, int TC_, int V_, int RL_, int RREG_>
 struct RegShape {
-    static constexpr int NN = NN_, PREC = 0, TC = TC_, VW = 4, V = V_, RL = RL_, RREG = RREG_, CL = CL_;
-    static_assert(CL == 1 || CL == NN / 2, "the u-step's blocks are one cluster");
+    static constexpr int NN = NN_, PREC = 0, TC = TC_, VW = 4, V = V_, RL = RL_, RREG = RREG_;
     static constexpr int N = NN * NN, THREADS = TC * RL, WARPS = THREADS / 32, WPR = TC / 32, CP = VW * V / 2;
     static_assert(TC * VW * V == N && TC % 32 == 0 && RREG % 4 == 0 && THREADS >= 96 && THREADS <= 512, "split");
     static constexpr int NP = NN / 2, GC = 2 * NN / 4, GG = THREADS / GC, WL = 3 * NN;
@@ -146,9 +139,7 @@ struct RegShape {
     static constexpr size_t O_FB = O_FA + NN * 8;
     static constexpr size_t O_TW = O_FB + NN * 8;
     static constexpr size_t O_RD = O_TW + NN * 8;
-    static constexpr size_t O_COLX = O_RD + 2 * NN * 4;                   // [2][n][2] words
-    static constexpr size_t O_ROWX = O_COLX + (CL > 1 ? 2 * NN * 16 : 0);  // [2][2][n/2][2] words
-    static constexpr size_t O_RED = O_ROWX + (CL > 1 ? 2 * NN * 16 : 0);
+    static constexpr size_t O_RED = O_RD + 2 * NN * 4;
     static constexpr size_t ROW_BYTES = (size_t)RED * 4 + 8;   // a row's warp sums, r and f
     static constexpr size_t LIMIT = 227 * 1024;
     static constexpr int XMAX = (int)((LIMIT - O_RED - 64 - RROWS * ROW_BYTES) / ((size_t)N * 4 + ROW_BYTES));
@@ -262,28 +253,8 @@ __device__ __forceinline__ void loop_ustep(const LoopArgs& q, int it)
     float2* fb = LOOP_AT(float2, S::O_FB);
     const float2* tw = LOOP_AT(float2, S::O_TW);
     const float* rdiv = LOOP_AT(float, S::O_RD);
-    constexpr bool HERE = S::CL > 1;   // column slots and rows through shared memory
-    uint64_t *colx, *rowx;             // of all blocks, or this block's
-    if constexpr (HERE) {
-        colx = LOOP_AT(uint64_t, S::O_COLX) + half * NN * 2;
-        rowx = LOOP_AT(uint64_t, S::O_ROWX) + half * NN * 2;
-    } else {
-        colx = q.colx + (size_t)half * NP * NN * 2;
-        rowx = q.rowx + (size_t)half * NN * NP * 2;
-    }
-    auto send_col = [&](int s, int r, float a, float b) {   // row r's entry of column slot s
-        if constexpr (HERE)
-            send2_to(colx + r * 2, s, a, b, tag);
-        else
-            send2(colx + ((size_t)s * NN + r) * 2, a, b, tag);
-    };
-    auto send_row = [&](int r, float a, float b) {          // this slot's entry of row r
-        if constexpr (HERE)
-            send2_to(rowx + ((r & 1) * NP + blk) * 2, r >> 1, a, b, tag);
-        else
-            send2(rowx + ((size_t)r * NP + blk) * 2, a, b, tag);
-    };
-    auto peek = [&](const uint64_t* p) { return HERE ? peek2_here(p) : peek2(p); };
+    uint64_t* colx = q.colx + (size_t)half * NP * NN * 2;
+    uint64_t* rowx = q.rowx + (size_t)half * NN * NP * 2;
     uint64_t* ubuf = q.ubuf + (size_t)half * N;
     if (lane == 0) st->pending = st->algo == 0 ? 1 : 0;   // u is about to move
     // a3: right-hand side of the two rows as one complex sequence
@@ -302,13 +273,14 @@ __device__ __forceinline__ void loop_ustep(const LoopArgs& q, int it)
     // half spectra of the two rows to the column slots' blocks
     for (int s = lane; s < NP; s += 32) {
         const float2 a = Z[s], b = Z[(NN - s) % NN];
+        uint64_t* dst = colx + ((size_t)s * NN + r0) * 2;
         if (s == 0) {
             const float2 n2 = Z[NN / 2];
-            send_col(s, r0, a.x, n2.x);
-            send_col(s, r0 + 1, a.y, n2.y);
+            send2(dst, a.x, n2.x, tag);
+            send2(dst + 2, a.y, n2.y, tag);
         } else {
-            send_col(s, r0, 0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-            send_col(s, r0 + 1, 0.5f * (a.y + b.y), -0.5f * (a.x - b.x));
+            send2(dst, 0.5f * (a.x + b.x), 0.5f * (a.y - b.y), tag);
+            send2(dst + 2, 0.5f * (a.y + b.y), -0.5f * (a.x - b.x), tag);
         }
     }
     __syncwarp();
@@ -316,14 +288,14 @@ __device__ __forceinline__ void loop_ustep(const LoopArgs& q, int it)
     {
         constexpr int K = (NN + 31) / 32;
         ulonglong2 v[K];
-        const uint64_t* src = HERE ? colx : colx + (size_t)blk * NN * 2;
+        const uint64_t* src = colx + (size_t)blk * NN * 2;
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            if (lane + 32 * k < NN) v[k] = peek(src + 2 * (lane + 32 * k));
+            if (lane + 32 * k < NN) v[k] = peek2(src + 2 * (lane + 32 * k));
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (lane + 32 * k < NN) {
-                v[k] = await2<HERE>(src + 2 * (lane + 32 * k), tag, v[k], waits);
+                v[k] = await2(src + 2 * (lane + 32 * k), tag, v[k], waits);
                 fa[lane + 32 * k] = make_float2(word_f(v[k].x), word_f(v[k].y));
             }
     }
@@ -347,24 +319,24 @@ __device__ __forceinline__ void loop_ustep(const LoopArgs& q, int it)
     }
     __syncwarp();
     const float2* Y = fft_warp<NN, true>(X, X == fa ? fb : fa, tw, lane);
-    for (int p = lane; p < NN; p += 32) send_row(p, Y[p].x, Y[p].y);
+    for (int p = lane; p < NN; p += 32) send2(rowx + ((size_t)p * NP + blk) * 2, Y[p].x, Y[p].y, tag);
     __syncwarp();
     // the rows' half spectra, packed for one inverse transform
     {
         constexpr int K = (NP + 31) / 32;
         ulonglong2 v[2][K];
-        const uint64_t* src = HERE ? rowx : rowx + (size_t)r0 * NP * 2;
+        const uint64_t* src = rowx + (size_t)r0 * NP * 2;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int k = 0; k < K; ++k)
-                if (lane + 32 * k < NP) v[h][k] = peek(src + 2 * (h * NP + lane + 32 * k));
+                if (lane + 32 * k < NP) v[h][k] = peek2(src + 2 * (h * NP + lane + 32 * k));
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int s = lane + 32 * k;
             if (s >= NP) continue;
-            const ulonglong2 vx = await2<HERE>(src + 2 * s, tag, v[0][k], waits);
-            const ulonglong2 vy = await2<HERE>(src + 2 * (NP + s), tag, v[1][k], waits);
+            const ulonglong2 vx = await2(src + 2 * s, tag, v[0][k], waits);
+            const ulonglong2 vy = await2(src + 2 * (NP + s), tag, v[1][k], waits);
             const float2 Xv = make_float2(word_f(vx.x), word_f(vx.y));
             const float2 Yv = make_float2(word_f(vy.x), word_f(vy.y));
             if (s == 0) {
@@ -923,23 +895,17 @@ __global__ void __maxnreg__(128) k_loop(const __grid_constant__ LoopArgs q)
     loop_end<S>(q, it);
 }
 
-template <int NN, int TC, int V, int RL, int RREG, int CL>
+template <int NN, int TC, int V, int RL, int RREG>
 __global__ void __launch_bounds__(TC * RL, 1) k_loop_reg(const __grid_constant__ LoopArgs q)
 {
-    using S = RegShape<NN, TC, V, RL, RREG, CL>;
+    using S = RegShape<NN, TC, V, RL, RREG>;
     LOOP_SMEM;
     volatile LoopState* st = LOOP_AT(LoopState, S::O_STATE);
     loop_begin<S>(q);
     uint64_t a[RREG][S::CP];
     const int lane_row = threadIdx.x / TC;
     reg_load_rows<S>(q, st->i0, st->nrows, lane_row, threadIdx.x - lane_row * TC, a, LOOP_AT(float, S::O_A));
-    if constexpr (CL > 1) {   // no word carries a tag yet, and no block sends before all are there
-        for (int i = threadIdx.x; i < 8 * NN; i += S::THREADS) LOOP_AT(uint64_t, S::O_COLX)[i] = 0ull;
-        cluster_arrive();
-        cluster_wait();
-    } else {
-        __syncthreads();
-    }
+    __syncthreads();
     int it = 0;
     while (true) {
         ++it;
@@ -953,10 +919,6 @@ __global__ void __launch_bounds__(TC * RL, 1) k_loop_reg(const __grid_constant__
         if (end) break;
     }
     loop_end<S>(q, it);
-    if constexpr (CL > 1) {   // no block leaves while another may still send to it
-        cluster_arrive();
-        cluster_wait();
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1029,25 +991,24 @@ static cudaError_t launch_loop_t(int grid, const LoopArgs& a, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------------------
-// Shapes with every row on chip: n -> (rows per block aimed at, TC, V, RL, RREG, CL).  Fewer threads
+// Shapes with every row on chip: n -> (rows per block aimed at, TC, V, RL, RREG).  Fewer threads
 // with more columns each leave the registers for A (8 rows of 16 columns at n = 64).  Measured
 // at n = 64, m = 1229: 256 x 16 columns 9.7 us, 512 x 8 9.6; n = 48: 288 x 8 8.0, 139 blocks of 5
-// rows instead of 87 9.0; n = 32, m = 307: 16, 32, 48, 64, 96 blocks 7.7, 7.3, 7.4, 7.5, 7.6.
+// rows instead of 87 9.0; n = 32: 39 blocks of 8 rows 7.3, 20 of 16 8.1.
 // ---------------------------------------------------------------------------
-#define TVCS_REG_TABLE(X)           \
-    X(16, 32, 64, 1, 4, 8, 8)       \
-    X(32, 12, 256, 1, 1, 12, 16)    \
-    X(48, 8, 288, 2, 1, 8, 1)       \
-    X(64, 8, 256, 4, 1, 8, 1)
+#define TVCS_REG_TABLE(X)     \
+    X(16, 32, 64, 1, 4, 8)    \
+    X(32, 8, 256, 1, 1, 8)    \
+    X(48, 8, 288, 2, 1, 8)    \
+    X(64, 8, 256, 4, 1, 8)
 
-template <int NN, int TC, int V, int RL, int RREG, int CL>
+template <int NN, int TC, int V, int RL, int RREG>
 static bool reg_configure_t()
 {
-    using S = RegShape<NN, TC, V, RL, RREG, CL>;
-    auto kernel = k_loop_reg<NN, TC, V, RL, RREG, CL>;
+    using S = RegShape<NN, TC, V, RL, RREG>;
+    auto kernel = k_loop_reg<NN, TC, V, RL, RREG>;
     int per = 0;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(S::RMAX)) != cudaSuccess ||
-        (CL > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, S::THREADS, S::smem(S::RMAX)) != cudaSuccess ||
         per < 1) {
         cudaGetLastError();
@@ -1058,55 +1019,21 @@ static bool reg_configure_t()
 
 bool reg_configure(int n)
 {
-#define X(NN, MR, TC, V, RL, RREG, CL) \
-    if (n == NN) return reg_configure_t<NN, TC, V, RL, RREG, CL>();
+#define X(NN, MR, TC, V, RL, RREG) \
+    if (n == NN) return reg_configure_t<NN, TC, V, RL, RREG>();
     TVCS_REG_TABLE(X)
 #undef X
     return false;
 }
 
-template <int NN, int TC, int V, int RL, int RREG, int CL>
-static void reg_config(int grid, int m, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr)
-{
-    using S = RegShape<NN, TC, V, RL, RREG, CL>;
-    cfg->gridDim = dim3(grid, 1, 1);
-    cfg->blockDim = dim3(S::THREADS, 1, 1);
-    cfg->dynamicSmemBytes = S::smem((m + grid - 1) / grid);
-    attr[0].id = cudaLaunchAttributeCooperative;   // the blocks wait for one another
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = CL;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg->attrs = attr;
-    cfg->numAttrs = CL > 1 ? 2 : 1;
-}
-
-template <int NN, int TC, int V, int RL, int RREG, int CL>
-static int reg_grid_t(int m, int mr, int num_sms)
-{
-    using S = RegShape<NN, TC, V, RL, RREG, CL>;
-    int g = std::min(num_sms / CL, (std::max(NN / 2, (m + mr - 1) / mr) + CL - 1) / CL) * CL;
-    if (CL > 1 && g > 0) {   // as many whole clusters as fit side by side
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[2];
-        reg_config<NN, TC, V, RL, RREG, CL>(CL, S::RMAX * CL, &cfg, attr);
-        cfg.gridDim = dim3(g, 1, 1);
-        cfg.attrs = attr + 1;
-        cfg.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, k_loop_reg<NN, TC, V, RL, RREG, CL>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
-        g = std::min(g, nc * CL);
-    }
-    return g >= NN / 2 && (m + g - 1) / g <= S::RMAX ? g : 0;
-}
-
 int reg_grid(int n, int m, int num_sms)
 {
-#define X(NN, MR, TC, V, RL, RREG, CL) \
-    if (n == NN) return reg_grid_t<NN, TC, V, RL, RREG, CL>(m, MR, num_sms);
+    if (num_sms < n / 2) return 0;
+#define X(NN, MR, TC, V, RL, RREG)                                              \
+    if (n == NN) {                                                              \
+        const int g = std::min(num_sms, std::max(n / 2, (m + MR - 1) / MR));    \
+        return (m + g - 1) / g <= RegShape<NN, TC, V, RL, RREG>::RMAX ? g : 0;  \
+    }
     TVCS_REG_TABLE(X)
 #undef X
     return 0;
@@ -1115,12 +1042,19 @@ int reg_grid(int n, int m, int num_sms)
 cudaError_t launch_loop_reg(int n, int grid, const LoopArgs& a, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
+    cfg.gridDim = dim3(grid, 1, 1);
     cfg.stream = s;
-#define X(NN, MR, TC, V, RL, RREG, CL)                                             \
-    if (n == NN) {                                                                 \
-        reg_config<NN, TC, V, RL, RREG, CL>(grid, a.m, &cfg, attr);                \
-        return cudaLaunchKernelEx(&cfg, k_loop_reg<NN, TC, V, RL, RREG, CL>, a);   \
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // the blocks wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+#define X(NN, MR, TC, V, RL, RREG)                                                    \
+    if (n == NN) {                                                                    \
+        using S = RegShape<NN, TC, V, RL, RREG>;                                      \
+        cfg.blockDim = dim3(S::THREADS, 1, 1);                                        \
+        cfg.dynamicSmemBytes = S::smem((a.m + grid - 1) / grid);                      \
+        return cudaLaunchKernelEx(&cfg, k_loop_reg<NN, TC, V, RL, RREG>, a);          \
     }
     TVCS_REG_TABLE(X)
 #undef X

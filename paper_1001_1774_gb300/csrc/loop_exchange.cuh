@@ -6,8 +6,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "common.cuh"
-
 namespace tvcs {
 
 __device__ __forceinline__ int fresh_tid()   // not kept from one section to the next
@@ -45,25 +43,6 @@ __device__ __forceinline__ bool has_tag(ulonglong2 v, uint32_t tag)
 
 __device__ __forceinline__ float word_f(uint64_t v) { return __uint_as_float((uint32_t)v); }
 
-// The same between the blocks of a cluster: the words lie in the reader's shared memory (p: this
-// block's address of the place; rank: the block it is meant for).
-__device__ __forceinline__ void send2_to(const uint64_t* p, int rank, float a, float b, uint32_t tag)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    asm volatile("st.relaxed.cluster.shared::cluster.v2.b64 [%0], {%1, %2};" ::"r"(r), "l"(tagged(a, tag)),
-                 "l"(tagged(b, tag))
-                 : "memory");
-}
-
-__device__ __forceinline__ ulonglong2 peek2_here(const uint64_t* p)
-{
-    ulonglong2 v;
-    asm volatile("ld.relaxed.cluster.shared::cta.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(smem_u32(p))
-                 : "memory");
-    return v;
-}
-
 // Bound of a block's waits, and its record that one gave up.
 struct Waits {
     long long budget;
@@ -71,15 +50,13 @@ struct Waits {
 };
 
 // The two words at p once both carry `tag` (v: a first look at them); whatever is there
-// when the budget runs out or another wait of the block has given up.  HERE: p is in this
-// block's shared memory.
-template <bool HERE = false>
+// when the budget runs out or another wait of the block has given up.
 __device__ __forceinline__ ulonglong2 await2(const uint64_t* p, uint32_t tag, ulonglong2 v, const Waits& w)
 {
     if (has_tag(v, tag)) return v;
     const long long t0 = clock64();
     for (;;) {
-        v = HERE ? peek2_here(p) : peek2(p);
+        v = peek2(p);
         if (has_tag(v, tag)) return v;
         if (*w.gave_up) return v;
         if (clock64() - t0 > w.budget) {
