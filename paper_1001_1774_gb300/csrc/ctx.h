@@ -91,11 +91,12 @@ struct tvcs_ctx {
     cudaGraphExec_t tail[16] = {};
     // the loop as one launch (n <= 96, stored A): blocks (0: the graphs above), whether A stays on
     // chip (launch_loop_reg); blocks of the power iteration's launch (0: a launch per product);
-    // exchange buffers, tags used so far
+    // exchange buffers (one array of exch_words words from ubuf on), the last tag used (take_tags)
     int loop_grid = 0;
     bool loop_reg = false;
     int power_grid = 0;
     uint64_t *ubuf = nullptr, *colx = nullptr, *rowx = nullptr, *nbuf = nullptr;
+    size_t exch_words = 0;
     uint32_t loop_tag = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool state_ready = false;

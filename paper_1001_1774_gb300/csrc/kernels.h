@@ -99,8 +99,9 @@ cudaError_t launch_greduce(const float* gpart, int P, int N, float* g, const Ctr
                            cudaStream_t s);
 
 // The whole iteration loop of one problem with a stored A, n <= 96, as one cooperative
-// launch (k_loop.cu).  Buffers of tagged words (zeroed once): ubuf 2 N, colx and rowx
-// 2 n/2 n 2, nbuf 2 n/2 4.  Iteration k of a launch uses tag tag0 + k; tags never repeat.
+// launch (k_loop.cu).  Buffers of tagged words (zeroed at first): ubuf 2 N, colx and rowx
+// 2 n/2 n 2, nbuf 2 n/2 4.  Iteration k of a launch uses tag tag0 + k, which no word carries
+// yet: the caller sees to it that tags never repeat (take_tags, tvcs_api.cu).
 struct LoopArgs {
     const unsigned char* P0;
     const unsigned char* P1;

@@ -325,6 +325,20 @@ tvcs_status init_state(tvcs_ctx* h, int init)
     return TVCS_OK;
 }
 
+// tag0 of a launch whose steps tag their words tag0 + 1 .. tag0 + steps.  A handle's tags only
+// grow, so that no word carries a tag that is still to come; before they would pass 2^32 - 1
+// the words are cleared (tag 0, which no step uses) and the tags start over.
+tvcs_status take_tags(tvcs_ctx* h, int steps, uint32_t* tag0)
+{
+    if ((uint32_t)steps > UINT32_MAX - h->loop_tag) {
+        CK(cudaMemsetAsync(h->ubuf, 0, sizeof(uint64_t) * h->exch_words, h->stream));
+        h->loop_tag = 0;
+    }
+    *tag0 = h->loop_tag;
+    h->loop_tag += (uint32_t)steps;
+    return TVCS_OK;
+}
+
 // The loop as one launch (k_loop.cu, k_dct_loop.cu).
 tvcs_status launch_iterations(tvcs_ctx* h, int iters)
 {
@@ -373,8 +387,7 @@ tvcs_status launch_iterations(tvcs_ctx* h, int iters)
     a.mu_over_tau = (float)(h->mu / h->tau);
     a.mu = (float)h->mu;
     a.iters = iters;
-    a.tag0 = h->loop_tag;
-    h->loop_tag += (uint32_t)iters;
+    CKS(take_tags(h, iters, &a.tag0));
     a.budget = budget_of(h);
     a.bar_extra = h->bar_extra;
     if (h->loop_reg)
@@ -462,8 +475,7 @@ tvcs_status power_tau(tvcs_ctx* h, int iters, double* tau_out)
         a.iters = iters;
         a.v0 = v0;
         a.xbuf = h->ubuf;
-        a.tag0 = h->loop_tag;
-        h->loop_tag += (uint32_t)iters;
+        CKS(take_tags(h, iters, &a.tag0));
         a.r2part = h->r2part;
         a.ctrl = h->ctrl;
         a.budget = budget_of(h);
@@ -621,10 +633,10 @@ tvcs_status create_impl(tvcs_ctx* h, const float* A, uint64_t seed, const int32_
     if (h->loop_grid || h->power_grid) {
         // ubuf, colx, rowx of 2 N words and nbuf of 4 n (k_loop.cu), or what k_power.cu wants,
         // in one zeroed array
-        size_t words = h->loop_grid ? 6 * N + 4 * (size_t)h->n : 0;
-        if (h->power_grid) words = std::max(words, power_words(h->n, h->power_grid));
-        CKS(alloc((void**)&h->ubuf, sizeof(uint64_t) * words));
-        CK(cudaMemsetAsync(h->ubuf, 0, sizeof(uint64_t) * words, h->stream));
+        h->exch_words = h->loop_grid ? 6 * N + 4 * (size_t)h->n : 0;
+        if (h->power_grid) h->exch_words = std::max(h->exch_words, power_words(h->n, h->power_grid));
+        CKS(alloc((void**)&h->ubuf, sizeof(uint64_t) * h->exch_words));
+        CK(cudaMemsetAsync(h->ubuf, 0, sizeof(uint64_t) * h->exch_words, h->stream));
         h->colx = h->ubuf + 2 * N;
         h->rowx = h->colx + 2 * N;
         h->nbuf = h->rowx + 2 * N;
