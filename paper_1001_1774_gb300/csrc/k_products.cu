@@ -42,7 +42,15 @@ constexpr size_t PROD_PF_BYTES = 1024 * 1024;
 // One block per SM (the ring fills shared memory at the larger sizes); the grid
 // leaves 16 SMs to the u-solve cluster of the same iteration, which runs there
 // while this kernel streams A.
-template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
+//
+// BIG: a block may have more than YMAX rows.  Up to that many, y (and the scales) of a block's
+// rows are fetched into shared memory at the start, so that no step waits on a global load
+// for them.  BIG: one thread a row fetches y with each step, into two sets of a step's rows, and
+// before the step's barrier: r may be stored over y (tvcs_apply_noalloc), so nobody may look for y
+// after it.  (Two kernels, because one that chose inside the step cost n = 128 up to 1 %: us an
+// iteration, binary32 52.0, bf16 56.4, fp8 48.1 where it read y of such blocks after the barrier,
+// 52.1, 56.3, 47.7 with the choice, 52.0, 56.0, 45.7 as two.)
+template <int PREC, int TC, int VW, int V, int RL, int RB, int NST, bool BIG>
 __global__ void __maxnreg__(128)
     k_products(const unsigned char* __restrict__ P0, const unsigned char* __restrict__ P1,
                const float* __restrict__ rscale, int m, const float* __restrict__ x,
@@ -132,10 +140,7 @@ __global__ void __maxnreg__(128)
     }
 
     // ---------------- consumers ----------------
-    // y (and the scales) of this block's rows, prefetched so that no step waits on a
-    // global load for them.
-    const bool in_smem = nrows <= S::YMAX;
-    if (in_smem) {
+    if constexpr (!BIG) {
         for (int i = tid; i < nrows; i += THREADS) sy[i] = y != nullptr ? y[i0 + i] : 0.f;
         if constexpr (PREC == 2)
             for (int i = tid; i < nrows; i += THREADS) ss[i] = rscale[i0 + i];
@@ -176,13 +181,14 @@ __global__ void __maxnreg__(128)
         const int li0 = s * RS + lane_row * RB;   // first row of this lane's step, in the block
         uint64_t a[RB][CP];
         float* rb = red + ((s & 1) * RS + lane_row * RB) * WPR;
+        [[maybe_unused]] float* yb = sy + (s & 1) * RS + lane_row * RB;
         float d[RB];
 #pragma unroll
         for (int b = 0; b < RB; ++b) {
             if (RS == 1 || li0 + b < nrows) {
                 const size_t row = (size_t)(lane_row * RB + b) * N;
                 float sc = 1.f;
-                if constexpr (PREC == 2) sc = in_smem ? ss[li0 + b] : rscale[i0 + li0 + b];
+                if constexpr (PREC == 2) sc = BIG ? rscale[i0 + li0 + b] : ss[li0 + b];
 #pragma unroll
                 for (int v = 0; v < V; ++v)
                     load_entries<PREC, VW>(sb + row * S::B0, sb + S::P1_OFF + row * S::B1,
@@ -209,6 +215,11 @@ __global__ void __maxnreg__(128)
         if ((tid & 31) == 0) {
 #pragma unroll
             for (int b = 0; b < RB; ++b) rb[b * WPR + warp_in_row] = d[b];
+        }
+        if constexpr (BIG) {
+            if (ltid == 0)
+                for (int b = 0; b < RB; ++b)
+                    if (li0 + b < nrows) yb[b] = y != nullptr ? y[i0 + li0 + b] : 0.f;
         }
         named_barrier(1, THREADS);   // the warps' parts are there, and nobody reads the stage any more
         // refill this slot with stage s + NST
@@ -240,7 +251,7 @@ __global__ void __maxnreg__(128)
 #pragma unroll
                 for (int w = 1; w < WPR; ++w) dot += rb[b * WPR + w];
             }
-            const float ri = dot - (in_smem ? sy[li] : (y != nullptr ? y[i0 + li] : 0.f));
+            const float ri = dot - (BIG ? yb[b] : sy[li]);
             if (ltid == 0) {
                 r[i0 + li] = ri;
                 r2 = ds_add(r2, ds_sq(ri));
@@ -408,18 +419,22 @@ static cudaError_t launch_prod_t(int grid, const ProdArgs& a, cudaStream_t s)
     cfg.attrs = attr;
     cfg.numAttrs = na;
     const int pf = (int)(PROD_PF_BYTES / S::STAGE);
-    return cudaLaunchKernelEx(&cfg, k_products<PREC, TC, VW, V, RL, RB, NST>, a.P0, a.P1, a.rscale,
-                              a.m, a.x, a.y, a.r, a.gpart, a.g_out, a.r2part, a.ctrl, a.mode,
-                              (cudaGraphConditionalHandle)a.cond, a.set_cond, a.budget, pf,
-                              a.bar_extra, a.host_err);
+    auto kernel = (a.m + grid - 1) / grid > S::YMAX ? k_products<PREC, TC, VW, V, RL, RB, NST, true>
+                                                    : k_products<PREC, TC, VW, V, RL, RB, NST, false>;
+    return cudaLaunchKernelEx(&cfg, kernel, a.P0, a.P1, a.rscale, a.m, a.x, a.y, a.r, a.gpart, a.g_out,
+                              a.r2part, a.ctrl, a.mode, (cudaGraphConditionalHandle)a.cond, a.set_cond,
+                              a.budget, pf, a.bar_extra, a.host_err);
 }
 
 template <int PREC, int TC, int VW, int V, int RL, int RB, int NST>
 static cudaError_t configure_t()
 {
     using S = ProdShape<PREC, TC, VW, V, RL, RB, NST>;
-    return cudaFuncSetAttribute(k_products<PREC, TC, VW, V, RL, RB, NST>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    for (auto kernel : {k_products<PREC, TC, VW, V, RL, RB, NST, false>, k_products<PREC, TC, VW, V, RL, RB, NST, true>}) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 //    precision, n, minimum rows per block, TC, VW, V, RL, RB, NST

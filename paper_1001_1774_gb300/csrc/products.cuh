@@ -19,7 +19,7 @@ struct ProdShape {
     static constexpr int B0 = PREC == 0 ? 4 : PREC == 1 ? 2 : 1, B1 = PREC == 0 ? 0 : 2;   // bytes per entry
     static constexpr size_t P1_OFF = (size_t)RS * N * B0;          // second plane in a stage
     static constexpr size_t STAGE = (size_t)RS * N * (B0 + B1);
-    static constexpr int YMAX = 1024;   // rows of y (and row scales) prefetched into shared memory
+    static constexpr int YMAX = 1024;   // most rows of a block whose y (and scales) are fetched at its start
     static constexpr size_t O_BAR = NST * STAGE;
     static constexpr size_t O_RED = O_BAR + ((NST * 8 + 15) / 16) * 16;         // [2][RS][WPR]
     static constexpr size_t O_DRED = O_RED + ((2 * RS * WPR * 4 + 15) / 16) * 16;   // [32] float2
@@ -30,6 +30,7 @@ struct ProdShape {
     static_assert(TC % 32 == 0 && THREADS <= 512, "row lanes must be whole warps");
     static_assert((N * B0) % 16 == 0, "TMA sizes are multiples of 16 bytes");
     static_assert(SMEM <= 227 * 1024, "shared memory");
+    static_assert(2 * RS <= YMAX, "y of two steps");
     static_assert(NST * STAGE >= (size_t)(RL - 1) * N * 4 && NST * STAGE >= (size_t)WARPS * 32 * 16,
                   "the ring doubles as scratch of the epilogue");
 };
