@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "kernels.h"
+#include "tuner_rule.h"
 
 namespace tvcs {
 
@@ -390,7 +391,8 @@ std::map<std::tuple<int, int, int, int>, std::pair<GemmShape, GemmShape>> g_gemm
 // Picks the launch shape of each GEMM (persistent blocks or pairs, and with it
 // the stream-K split of its tiles x K-blocks) by timing every candidate, GEMM
 // and fix-up together, over five launches each (median), on the handle's own
-// operands; cached per device and (m, n).  opt.autotune = 0 keeps one block
+// operands; cached per device and (m, n).  A shape takes the place of an earlier one only where
+// it is faster beyond the noise (tuner_rule.h).  opt.autotune = 0 keeps one block
 // per SM; a shape set through tvcs_test_gemm_shape takes precedence.  A
 // different split regroups the K sums of a tile, so results agree to binary32
 // rounding with the default shape, not bitwise.
@@ -423,8 +425,9 @@ tvcs_status tune_gemms(tvcs_ctx* h, int count)
             const long long budget = h->opt.timeout_cycles > 0 ? h->opt.timeout_cycles : (1LL << 31);
             for (int which = 0; which < 2; ++which) {
                 const int M = which == 0 ? h->m : h->N, K = which == 0 ? h->N : h->m;
-                float best = -1.f;
-                for (GemmShape g : gemm_shape_candidates(h->num_sms, b->pair_clusters, nt)) {
+                const std::vector<GemmShape> shapes = gemm_shape_candidates(h->num_sms, b->pair_clusters, nt);
+                std::vector<float> times;
+                for (const GemmShape& g : shapes) {
                     GemmPlan p;
                     gemm_plan(M, K, g.grid, &p, g.pair != 0, nt);
                     int *tsb = nullptr, *ss = nullptr;
@@ -455,11 +458,9 @@ tvcs_status tune_gemms(tvcs_ctx* h, int count)
                     cudaFree(tsb);
                     cudaFree(ss);
                     std::sort(t, t + 5);
-                    if (best < 0.f || t[2] < best) {
-                        best = t[2];
-                        (which == 0 ? g1 : g2) = g;
-                    }
+                    times.push_back(t[2]);
                 }
+                (which == 0 ? g1 : g2) = shapes[tuned_shape(times.data(), times.size())];
             }
             std::lock_guard<std::mutex> lk(g_gemm_tune_mutex);
             g_gemm_shapes[{h->dev, h->m, h->N, nt}] = {g1, g2};
