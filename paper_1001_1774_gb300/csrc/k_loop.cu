@@ -924,7 +924,8 @@ __global__ void __launch_bounds__(TC * RL, 1) k_loop_reg(const __grid_constant__
 // ---------------------------------------------------------------------------
 // Shape table: (precision, n) -> (TC, VW, V, RL, RB, RP, NPC), rows a block takes at least.
 // The blocks are at least the n/2 of the u-step and at most one per SM.
-// (Up to 64 x 64 only what does not fit on chip comes here: m > 3192 at n = 64, 4712 at 48, 8000 at 32.)
+// (Up to 64 x 64 only what does not fit on chip comes here: on 152 SMs m > 3192 at n = 64, 4712 at
+// 48, 9272 at 32, 37544 at 16.)
 // ---------------------------------------------------------------------------
 //    precision, n, minimum rows per block, TC, VW, V, RL, RB, RP, NPC
 #define TVCS_LOOP_TABLE(X)                   \
