@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 import numpy as np
 
@@ -114,18 +115,19 @@ def _check(status: int) -> int:
     return status
 
 
-try:
-    import torch as _torch
-except ImportError:   # numpy arrays only
-    _torch = None
+def _torch():
+    """torch where the program has imported it (there are no tensors otherwise), else None."""
+    t = sys.modules.get("torch")
+    return t if hasattr(t, "Tensor") else None
 
 
 def _ptr(x, count: int | None = None, writable: bool = False):
     """Raw pointer of a contiguous float32 torch tensor or numpy array (host or device)."""
     if x is None:
         return None
-    if _torch is not None and isinstance(x, _torch.Tensor):
-        if x.dtype != _torch.float32 or not x.is_contiguous():
+    torch = _torch()
+    if torch is not None and isinstance(x, torch.Tensor):
+        if x.dtype != torch.float32 or not x.is_contiguous():
             raise TypeError("expected a contiguous float32 tensor")
         if count is not None and x.numel() != count:
             raise ValueError("expected %d elements, got %d" % (count, x.numel()))
@@ -146,15 +148,16 @@ def _ready(*arrays) -> None:
     wait for other streams.  Before a call that reads or writes torch CUDA tensors,
     finish the work queued on torch's current stream of each device involved (the
     tensors' producers, and pending readers of output buffers): once per device."""
-    if _torch is None:
+    torch = _torch()
+    if torch is None:
         return
     devs = set()
     for a in arrays:
         for x in (a if isinstance(a, (list, tuple)) else (a,)):
-            if isinstance(x, _torch.Tensor) and x.is_cuda:
+            if isinstance(x, torch.Tensor) and x.is_cuda:
                 devs.add(x.get_device())
     for d in devs:
-        _torch.cuda.current_stream(d).synchronize()
+        torch.cuda.current_stream(d).synchronize()
 
 
 def tvcs_default_options() -> tvcs_options:
