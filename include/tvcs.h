@@ -31,6 +31,11 @@
  *    The handle's stream does not wait for other streams: device arrays
  *    written (or still read) by work on another stream must be complete when
  *    the call is made, unless that stream is the handle's stream.
+ *  - Handles may be used by different host threads at the same time, each on its
+ *    stream.  The loop of a run that is one launch (tvcs_options.host_loop) holds
+ *    up to every SM until the run ends: other work on the device, another
+ *    handle's calls included, may wait for the whole run, not for one iteration.
+ *    host_loop = 1 gives the SMs back after every kernel.
  *  - Errors: a negative tvcs_status, with a message for tvcs_last_error().
  *    No call aborts, throws or exits.  Arguments are validated before any
  *    device work, so invalid arguments never reach a kernel.

@@ -34,6 +34,11 @@
 // reduction and a block barrier in series; from registers all rows share one of each.)  At
 // n = 128 k_loop measured 52.5 us against 52.1 (u-solve and exchanges take 13 us in which L2 cannot
 // hold more of A than the row order already keeps there), so that size keeps the chain.
+//
+// What it costs others: the launch holds its SMs (all of them at n = 96 and at n = 64 from m = 1209
+// on) for the whole run, where the chain gave them back every iteration.  Two threads with a
+// handle each, ms a call: 64 x 64 (m = 1229), 300 iterations, alone 3.3 (chain 4.6), both at once
+// 6.5 (6.1); 64 x 64, 20 iterations, next to runs of 300 at 96 x 96 5.1 (0.73).
 #include <cuda_runtime.h>
 
 #include <algorithm>
