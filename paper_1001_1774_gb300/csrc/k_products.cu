@@ -437,11 +437,13 @@ static cudaError_t configure_t()
     return cudaSuccess;
 }
 
+// (n = 48, binary32: 8 rows a step in two row lanes; 4 rows on 384 x 6 columns were slower from
+// m = 1152 on: 10.2, 14.3, 43.8 us a launch at m = 1152, 4700, 20000, here 9.8, 12.3, 36.8.)
 //    precision, n, minimum rows per block, TC, VW, V, RL, RB, NST
 #define TVCS_PROD_TABLE(X)                \
     X(0, 16, 8, 64, 4, 1, 8, 2, 4)        \
     X(0, 32, 4, 256, 4, 1, 2, 4, 4)       \
-    X(0, 48, 4, 384, 2, 3, 1, 4, 4)       \
+    X(0, 48, 4, 192, 4, 3, 2, 4, 3)       \
     X(0, 64, 2, 512, 4, 2, 1, 4, 3)       \
     X(0, 96, 1, 512, 2, 9, 1, 2, 3)       \
     X(0, 128, 1, 512, 4, 8, 1, 1, 3)      \
