@@ -115,17 +115,25 @@ def _check(status: int) -> int:
     return status
 
 
-def _torch():
-    """torch where the program has imported it (there are no tensors otherwise), else None."""
+_torch = None
+
+
+def _find_torch():
+    """torch where the program has imported it (there are no tensors otherwise), else None.
+    Kept once found: a call looks at up to two arrays an image, and a search for each cost
+    0.1 us an array (256 images of 64 x 64, one iteration: 1.49 -> 1.54 ms a batch)."""
+    global _torch
     t = sys.modules.get("torch")
-    return t if hasattr(t, "Tensor") else None
+    if hasattr(t, "Tensor"):
+        _torch = t
+    return _torch
 
 
 def _ptr(x, count: int | None = None, writable: bool = False):
     """Raw pointer of a contiguous float32 torch tensor or numpy array (host or device)."""
     if x is None:
         return None
-    torch = _torch()
+    torch = _torch if _torch is not None else _find_torch()
     if torch is not None and isinstance(x, torch.Tensor):
         if x.dtype != torch.float32 or not x.is_contiguous():
             raise TypeError("expected a contiguous float32 tensor")
@@ -148,7 +156,7 @@ def _ready(*arrays) -> None:
     wait for other streams.  Before a call that reads or writes torch CUDA tensors,
     finish the work queued on torch's current stream of each device involved (the
     tensors' producers, and pending readers of output buffers): once per device."""
-    torch = _torch()
+    torch = _torch if _torch is not None else _find_torch()
     if torch is None:
         return
     devs = set()

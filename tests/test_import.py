@@ -29,3 +29,21 @@ def test_the_binding_works_where_torch_does_not_load(tmp_path, error):
     env = dict(os.environ, PYTHONPATH=os.pathsep.join([str(tmp_path), ROOT]))
     p = subprocess.run([sys.executable, "-c", PROGRAM], env=env, cwd=str(tmp_path), capture_output=True, text=True)
     assert p.returncode == 0 and p.stdout.strip() == "ok", p.stderr
+
+
+def test_torch_imported_after_the_binding_is_found():
+    pytest.importorskip("torch")
+    program = PROGRAM + """
+import torch
+t = torch.zeros(4)
+for _ in range(2):
+    assert tv._ptr(t, 4).value == t.data_ptr()
+    assert tv._ptr(a, 4).value == a.ctypes.data
+    try:
+        tv._ptr(t.double())
+    except TypeError:
+        print("tensor")
+"""
+    p = subprocess.run([sys.executable, "-c", program], env=dict(os.environ, PYTHONPATH=ROOT), cwd=ROOT,
+                       capture_output=True, text=True)
+    assert p.returncode == 0 and p.stdout.split() == ["ok", "tensor", "tensor"], p.stderr
