@@ -390,7 +390,7 @@ std::map<std::tuple<int, int, int, int>, std::pair<GemmShape, GemmShape>> g_gemm
 
 // Picks the launch shape of each GEMM (persistent blocks or pairs, and with it
 // the stream-K split of its tiles x K-blocks) by timing every candidate, GEMM
-// and fix-up together, over five launches each (median), on the handle's own
+// and fix-up together, over five launches or three groups of launches each (median), on the handle's own
 // operands; cached per device and (m, n).  A shape takes the place of an earlier one only where
 // it is faster beyond the noise (tuner_rule.h).  opt.autotune = 0 keeps one block
 // per SM; a shape set through tvcs_test_gemm_shape takes precedence.  A
@@ -425,6 +425,7 @@ tvcs_status tune_gemms(tvcs_ctx* h, int count)
             const long long budget = h->opt.timeout_cycles > 0 ? h->opt.timeout_cycles : (1LL << 31);
             for (int which = 0; which < 2; ++which) {
                 const int M = which == 0 ? h->m : h->N, K = which == 0 ? h->N : h->m;
+                const int launches = tuner_launches(M, K), reps = launches > 1 ? 3 : 5;
                 const std::vector<GemmShape> shapes = gemm_shape_candidates(h->num_sms, b->pair_clusters, nt);
                 std::vector<float> times;
                 for (const GemmShape& g : shapes) {
@@ -433,20 +434,22 @@ tvcs_status tune_gemms(tvcs_ctx* h, int count)
                     int *tsb = nullptr, *ss = nullptr;
                     BCKS(upload_plan(p, &tsb, &ss, s));
                     float t[5];
-                    for (int rep = -1; rep < 5; ++rep) {
+                    for (int rep = -1; rep < reps; ++rep) {
                         if (rep >= 0) BCK(cudaEventRecord(h->ev0, s));
-                        if (which == 0) {
-                            launch_gemm(&b->mAh, &b->mAl, &b->mUh, &b->mUl, p, b->ws, b->bctrl, 0,
-                                        budget, s, count);
-                            launch_gemm_fixup(b->ws, tsb, ss, h->m, p.tiles_m, p.nt * 256, count, b->F, h->m,
-                                              b->R, h->m, b->Rh, b->Rl, b->mpad, b->r2part, b->bctrl,
-                                              0, s);
-                        } else {
-                            launch_gemm(&b->mAth, &b->mAtl, &b->mRh, &b->mRl, p, b->ws, b->bctrl, 0,
-                                        budget, s, count);
-                            launch_gemm_fixup(b->ws, tsb, ss, h->N, p.tiles_m, p.nt * 256, count, nullptr, 0,
-                                              b->G, h->N, nullptr, nullptr, 0, nullptr, b->bctrl, 0,
-                                              s);
+                        for (int k = 0; k < (rep < 0 ? 1 : launches); ++k) {
+                            if (which == 0) {
+                                launch_gemm(&b->mAh, &b->mAl, &b->mUh, &b->mUl, p, b->ws, b->bctrl, 0,
+                                            budget, s, count);
+                                launch_gemm_fixup(b->ws, tsb, ss, h->m, p.tiles_m, p.nt * 256, count, b->F, h->m,
+                                                  b->R, h->m, b->Rh, b->Rl, b->mpad, b->r2part, b->bctrl,
+                                                  0, s);
+                            } else {
+                                launch_gemm(&b->mAth, &b->mAtl, &b->mRh, &b->mRl, p, b->ws, b->bctrl, 0,
+                                            budget, s, count);
+                                launch_gemm_fixup(b->ws, tsb, ss, h->N, p.tiles_m, p.nt * 256, count, nullptr, 0,
+                                                  b->G, h->N, nullptr, nullptr, 0, nullptr, b->bctrl, 0,
+                                                  s);
+                            }
                         }
                         if (rep >= 0) {
                             BCK(cudaEventRecord(h->ev1, s));
@@ -457,8 +460,8 @@ tvcs_status tune_gemms(tvcs_ctx* h, int count)
                     BCKS(sync_check(h, "tuning the batched GEMMs"));
                     cudaFree(tsb);
                     cudaFree(ss);
-                    std::sort(t, t + 5);
-                    times.push_back(t[2]);
+                    std::sort(t, t + reps);
+                    times.push_back(t[reps / 2]);
                 }
                 (which == 0 ? g1 : g2) = shapes[tuned_shape(times.data(), times.size())];
             }
