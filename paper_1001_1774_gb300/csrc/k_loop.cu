@@ -30,6 +30,8 @@
 //   n = 16 (m = 77) 9.6 -> 6.7 -> 4.8, n = 32 (307) 11.7 -> 7.8 -> 7.3, n = 48 (691) 12.5 -> 8.7 ->
 //   8.0, n = 64 (1229) 14.75 -> 11.4 -> 9.7 (2048: 13.2 -> 10.0; fp8, 1229: 13.8 -> 9.7), n = 96
 //   (921) 17.0 -> 16.3, n = 96 (2765) 23.7 -> 23.3.
+// (k_loop_reg varies by where the exchange buffers lie on the two dies: over devices and handles
+// n = 16 4.8-6.1, n = 32 6.0-9.3, n = 48 8.0-9.0, n = 64 9.2-12.5.)
 // (From the ring a pass over 9 rows took three steps of 1.3 us, each a wait, a decode, a warp
 // reduction and a block barrier in series; from registers all rows share one of each.)  At
 // n = 128 k_loop measured 52.5 us against 52.1 (u-solve and exchanges take 13 us in which L2 cannot
